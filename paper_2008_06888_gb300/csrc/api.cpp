@@ -50,6 +50,7 @@ struct tn_ctx {
   char *d_arena = nullptr;
   int64_t arena_cap = 0;
   std::unique_ptr<Program> prog[3];
+  std::unique_ptr<Program> prog_sat;   // counts in one plane of exact 64-bit integers
   int prog_P = 0, prog_rb = 8;
   bool have_state = false;
   bool fwd_done = false;   // tn_forward ran last; its checkpoints are live
@@ -180,10 +181,11 @@ tn_status ensure_device(tn_ctx *ctx) {
   return TN_OK;
 }
 
-tn_status get_program(tn_ctx *ctx, ProgMode mode, int P, Program **out, int rb = 8) {
+tn_status get_program(tn_ctx *ctx, ProgMode mode, int P, Program **out, int rb = 8,
+                      bool sat = false) {
   if (!ctx->ordered) return fail(ctx, TN_ESTATE, "tn_order has not been called");
-  std::unique_ptr<Program> &slot = ctx->prog[mode];
-  if (!slot || (mode == PM_COUNT && (ctx->prog_P != P || ctx->prog_rb != rb))) {
+  std::unique_ptr<Program> &slot = sat ? ctx->prog_sat : ctx->prog[mode];
+  if (!slot || (mode == PM_COUNT && !sat && (ctx->prog_P != P || ctx->prog_rb != rb))) {
     if (slot) free_program(slot.get());
     slot.reset(new Program());
     int64_t seg = 0;
@@ -205,7 +207,7 @@ tn_status get_program(tn_ctx *ctx, ProgMode mode, int P, Program **out, int rb =
     }
     std::string err;
     if (!build_program(ctx->net, ctx->plan, mode, ctx->dt, mode == PM_COUNT ? P : 0, seg,
-                       slot.get(), &err, mode == PM_COUNT ? rb : 8)) {
+                       slot.get(), &err, mode == PM_COUNT ? rb : 8, sat)) {
       slot.reset();
       return fail(ctx, TN_EINVAL, err);
     }
@@ -225,7 +227,7 @@ tn_status get_program(tn_ctx *ctx, ProgMode mode, int P, Program **out, int rb =
       CK(cudaMemcpy(p.d_chain_traces, p.chain_traces.data(),
                     p.chain_traces.size() * sizeof(ChainTrace), cudaMemcpyHostToDevice));
     }
-    if (mode == PM_COUNT) {
+    if (mode == PM_COUNT && !sat) {
       ctx->prog_P = P;
       ctx->prog_rb = rb;
     }
@@ -311,6 +313,7 @@ tn_status run_ops(tn_ctx *ctx, Program &p, int op_begin, int op_end, cudaStream_
   ps.r32 = p.rbytes == 4;
   for (int i = 0; i < TN_MAX_PRIMES; ++i) ps.c[i] = ps.r32 ? kPrime31C[i] : kPrimeC[i];
   if (p.pass_prime) ps.c[0] = ctx->pass_c;   // one 31-bit prime per pass
+  if (p.sat) ps.c[0] = 0;                    // saturating counts
   auto X = [&](const Loc &l) -> void * { return l.buf < 0 ? nullptr : ar + abs_off(p, l); };
   auto Nn = [&](const Loc &l) -> uint64_t * {
     return l.buf < 0 ? nullptr : (uint64_t *)(ar + p.bufs[l.buf].off + l.noff);
@@ -559,15 +562,17 @@ tn_status ensure_batch(tn_ctx *ctx, int B) {
   return TN_OK;
 }
 
+// ids (optional): the B instances are ids[0..B) of the arrays J and h
 tn_status batch_setup(tn_ctx *ctx, int B, const float *J, const float *h, int on_device,
-                      ProgMode mode, int P, Program **out, RunArgs *ra, int rb = 8) {
+                      ProgMode mode, int P, Program **out, RunArgs *ra, int rb = 8,
+                      bool sat = false, const int *ids = nullptr) {
   const Net &n = ctx->net;
   if (B < 1) return fail(ctx, TN_EINVAL, "batch size must be >= 1");
   if (n.m > 0 && !J) return fail(ctx, TN_EINVAL, "J is NULL");
   const bool fields = !n.h.empty();
   if (fields && !h) return fail(ctx, TN_EINVAL, "the instance has fields: h is required");
   if (!fields && h) return fail(ctx, TN_EINVAL, "the instance was built without fields");
-  if (!on_device && ctx->dt == DT_I32) {
+  if (!on_device && ctx->dt == DT_I32 && !ids) {
     for (int64_t i = 0; i < (int64_t)B * n.m; ++i)
       if (std::nearbyint(J[i]) != J[i] || !(std::fabs(J[i]) < (float)(1 << 20)))
         return fail(ctx, TN_EINVAL, "INT32 context needs integral J");
@@ -579,13 +584,24 @@ tn_status batch_setup(tn_ctx *ctx, int B, const float *J, const float *h, int on
   tn_status s = ensure_device(ctx);
   if (s != TN_OK) return s;
   Program *p;
-  if ((s = get_program(ctx, mode, P, &p, rb)) != TN_OK) return s;
+  if ((s = get_program(ctx, mode, P, &p, rb, sat)) != TN_OK) return s;
   const int64_t stride = batch_stride(*p);
   if ((s = ensure_arena(ctx, stride * B)) != TN_OK) return s;
   if ((s = ensure_batch(ctx, B)) != TN_OK) return s;
   const cudaMemcpyKind kind = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
-  if (n.m) CK(cudaMemcpyAsync(ctx->d_Jb, J, (size_t)B * n.m * sizeof(float), kind, ctx->stream));
-  if (h) CK(cudaMemcpyAsync(ctx->d_hb, h, (size_t)B * n.n * sizeof(float), kind, ctx->stream));
+  if (!ids) {
+    if (n.m) CK(cudaMemcpyAsync(ctx->d_Jb, J, (size_t)B * n.m * sizeof(float), kind, ctx->stream));
+    if (h) CK(cudaMemcpyAsync(ctx->d_hb, h, (size_t)B * n.n * sizeof(float), kind, ctx->stream));
+  } else {
+    for (int b = 0; b < B; ++b) {
+      if (n.m)
+        CK(cudaMemcpyAsync(ctx->d_Jb + (size_t)b * n.m, J + (size_t)ids[b] * n.m,
+                           n.m * sizeof(float), kind, ctx->stream));
+      if (h)
+        CK(cudaMemcpyAsync(ctx->d_hb + (size_t)b * n.n, h + (size_t)ids[b] * n.n,
+                           n.n * sizeof(float), kind, ctx->stream));
+    }
+  }
   ctx->fwd_done = false;
   ra->bt.B = B;
   ra->bt.ib = stride;
@@ -642,6 +658,21 @@ CountRep count_rep(int n_primes) {
   return r;
 }
 
+// Counts below 2^64 - 1 need no residues: one 8-byte plane holds them exactly,
+// 4 + 8 bytes per element instead of 4 + 28 (mixed +-J batches of side 8..20: 192
+// instances in @@ ms instead of 46.6), and saturates where they do not fit; such an
+// instance is run again with the residue planes.  Contexts whose counts are likely to
+// be larger start there: +-J glasses have up to about 0.105 bits of ground-state
+// entropy per spin without fields (square lattices; 3-regular and chimera graphs less),
+// Max-2-SAT formulas about 0.35 bits per variable, so 64 bits hold up to some 600 spins
+// without and 180 with fields.  TN_COUNT_RESIDUES keeps the residue planes.
+bool sat_first(const tn_ctx *ctx) {
+  for (const char *v : {"TN_COUNT_RESIDUES", "TN_COUNT_61", "TN_COUNT_PASSES"})
+    if (std::getenv(v)) return false;
+  return ctx->net.n <= (ctx->net.h.empty() ? 600 : 180) || ctx->dt == DT_F32;
+}
+constexpr uint64_t kSaturated = ~0ull;
+
 // exact count from residues res[i] modulo rep.primes[i] (the last one the witness)
 tn_status count_from_residues(tn_ctx *ctx, const std::vector<uint64_t> &res, const CountRep &rep,
                               std::vector<uint64_t> *v) {
@@ -658,6 +689,14 @@ tn_status finish_count(tn_ctx *ctx, const std::vector<uint64_t> &res,
                        double *ln_count);
 tn_status count_in_passes(tn_ctx *ctx, int n_primes, uint64_t *limbs, int32_t *n_limbs,
                           double *ln_count, double *E);
+
+// the residues of an exact count: the primes' range and witness apply to it as to a
+// count that was kept in residues
+std::vector<uint64_t> residues_of(uint64_t v, const CountRep &rep) {
+  std::vector<uint64_t> r;
+  for (uint64_t p : rep.primes) r.push_back(v % p);
+  return r;
+}
 
 }  // namespace
 
@@ -812,6 +851,8 @@ tn_status tn_order(tn_ctx *ctx, int32_t method, const int32_t *seq, int32_t seq_
   }
   if (ctx->prog_pass) free_program(ctx->prog_pass.get());
   ctx->prog_pass.reset();
+  if (ctx->prog_sat) free_program(ctx->prog_sat.get());
+  ctx->prog_sat.reset();
   ctx->plan = p;
   ctx->ordered = true;
   ctx->have_state = false;
@@ -955,6 +996,23 @@ tn_status tn_count(tn_ctx *ctx, int32_t n_primes, uint64_t *limbs, int32_t *n_li
   Program *p;
   const bool force_passes = std::getenv("TN_COUNT_PASSES") != nullptr;
   if (force_passes) return count_in_passes(ctx, n_primes, limbs, n_limbs, ln_count, E);
+  if (sat_first(ctx)) {
+    s = get_program(ctx, PM_COUNT, 1, &p, 8, true);
+    if (s != TN_OK && s != TN_ENOMEM) return s;
+    if (s == TN_OK) {
+      if ((s = run_program(ctx, *p)) != TN_OK) return s;
+      char raw[4];
+      uint64_t v = 0;
+      const char *base = ctx->d_arena + p->bufs[p->root.buf].off;
+      CK(cudaMemcpyAsync(raw, base + p->root.xoff, 4, cudaMemcpyDeviceToHost, ctx->stream));
+      CK(cudaMemcpyAsync(&v, base + p->root.noff, 8, cudaMemcpyDeviceToHost, ctx->stream));
+      CK(cudaStreamSynchronize(ctx->stream));
+      if (v != kSaturated) {
+        if (E) *E = root_energy(ctx, raw);
+        return finish_count(ctx, residues_of(v, rep), rep.primes, limbs, n_limbs, ln_count);
+      }
+    }
+  }
   s = get_program(ctx, PM_COUNT, rep.P, &p, rep.rb);
   if (s == TN_ENOMEM) {
     // the residue planes do not fit: one 31-bit prime per pass
@@ -1130,16 +1188,19 @@ tn_status pinned_stage(tn_ctx *ctx, size_t bytes, char **out) {
 }
 
 // E, counts and statuses of B instances from their staged root values (raw:
-// 4 bytes each) and residues (res[i * B + b], plane i, the last the witness).
+// 4 bytes each) and residues (res[i * B + b], plane i, the last the witness) or, with
+// sat, exact counts (res[b]; saturated instances are left out).
 tn_status finish_counts(tn_ctx *ctx, int B, const CountRep &rep, const char *raw,
                         const uint64_t *res, uint64_t *limbs, int32_t limbs_per, double *E,
-                        int32_t *status) {
+                        int32_t *status, bool sat = false) {
   const int P = rep.P;
   tn_status first = TN_OK;
   for (int b = 0; b < B; ++b) {
+    if (sat && res[b] == kSaturated) continue;
     if (E) E[b] = root_energy(ctx, raw + 4 * b);
     std::vector<uint64_t> r(P), v;
-    for (int i = 0; i < P; ++i) r[i] = res[(size_t)i * B + b];
+    if (sat) r = residues_of(res[b], rep);
+    else for (int i = 0; i < P; ++i) r[i] = res[(size_t)i * B + b];
     tn_status sb = count_from_residues(ctx, r, rep, &v);
     if (sb == TN_OK && (int)v.size() > limbs_per) {
       sb = TN_EINVAL;
@@ -1151,6 +1212,45 @@ tn_status finish_counts(tn_ctx *ctx, int B, const CountRep &rep, const char *raw
     if (sb != TN_OK && first == TN_OK) first = sb;
   }
   return first;
+}
+
+tn_status stage_results(tn_ctx *ctx, const Program &p, int B, int P, char *raw, uint64_t *res);
+
+// E, counts and statuses of the instances ids[0..K) of a batch (arrays of the whole
+// batch), counted with the residue planes of `rep`.  Returns whether the run itself
+// worked (else its error is their status).
+tn_status count_residues(tn_ctx *ctx, const std::vector<int> &ids, const float *J, const float *h,
+                         int on_device, const CountRep &rep, uint64_t *limbs, int32_t limbs_per,
+                         double *E, int32_t *status) {
+  const int K = (int)ids.size();
+  Program *p;
+  RunArgs ra;
+  tn_status s = batch_setup(ctx, K, J, h, on_device, PM_COUNT, rep.P, &p, &ra, rep.rb, false,
+                            ids.data());
+  if (s == TN_OK) s = run_program(ctx, *p, 0, -1, ra);
+  std::vector<char> raw((size_t)K * 4);
+  std::vector<uint64_t> res((size_t)rep.P * K), lk((size_t)K * limbs_per);
+  if (s == TN_OK) s = stage_results(ctx, *p, K, rep.P, raw.data(), res.data());
+  if (s == TN_OK && cudaStreamSynchronize(ctx->stream) != cudaSuccess)
+    s = fail(ctx, TN_ECUDA, "counting with residue planes failed");
+  std::vector<double> Ek(K);
+  std::vector<int32_t> sk(K, s);
+  if (s == TN_OK)
+    finish_counts(ctx, K, rep, raw.data(), res.data(), lk.data(), limbs_per, Ek.data(), sk.data());
+  for (int k = 0; k < K; ++k) {
+    std::copy(lk.begin() + (size_t)k * limbs_per, lk.begin() + (size_t)(k + 1) * limbs_per,
+              limbs + (int64_t)ids[k] * limbs_per);
+    if (E) E[ids[k]] = Ek[k];
+    status[ids[k]] = sk[k];
+  }
+  return s;
+}
+
+// the first status of a batch that is not TN_OK
+tn_status first_of(const int32_t *status, int B) {
+  for (int b = 0; b < B; ++b)
+    if (status[b] != TN_OK) return (tn_status)status[b];
+  return TN_OK;
 }
 
 // queue the copies of B roots (and P residue planes) of a program's batch to host
@@ -1180,17 +1280,26 @@ tn_status tn_count_batch(tn_ctx *ctx, int32_t B, const float *J, const float *h,
     return fail(ctx, TN_EINVAL, "n_primes must be in [1, 8]");
   if (!limbs || limbs_per < 1) return fail(ctx, TN_EINVAL, "limbs buffer missing");
   const CountRep rep = count_rep(n_primes);
-  const int P = rep.P;
+  const bool sat = sat_first(ctx);
+  const int P = sat ? 1 : rep.P;
   Program *p;
   RunArgs ra;
-  tn_status s = batch_setup(ctx, B, J, h, on_device, PM_COUNT, P, &p, &ra, rep.rb);
+  tn_status s = batch_setup(ctx, B, J, h, on_device, PM_COUNT, P, &p, &ra, sat ? 8 : rep.rb, sat);
   if (s != TN_OK) return s;
   if ((s = run_program(ctx, *p, 0, -1, ra)) != TN_OK) return s;
   std::vector<char> raw((size_t)B * 4);
   std::vector<uint64_t> res((size_t)P * B);
   if ((s = stage_results(ctx, *p, B, P, raw.data(), res.data())) != TN_OK) return s;
   CK(cudaStreamSynchronize(ctx->stream));
-  return finish_counts(ctx, B, rep, raw.data(), res.data(), limbs, limbs_per, E, status);
+  std::vector<int32_t> own(status ? 0 : B, TN_OK);
+  if (!status) status = own.data();
+  s = finish_counts(ctx, B, rep, raw.data(), res.data(), limbs, limbs_per, E, status, sat);
+  std::vector<int> over;
+  for (int b = 0; sat && b < B; ++b)
+    if (res[b] == kSaturated) over.push_back(b);
+  if (over.empty()) return s;
+  s = count_residues(ctx, over, J, h, on_device, rep, limbs, limbs_per, E, status);
+  return s != TN_OK ? s : first_of(status, B);
 }
 
 tn_status tn_batch_run(int32_t B, tn_ctx *const *ctxs, double *E, uint64_t *limbs,
@@ -1262,7 +1371,7 @@ tn_status tn_batch_run(int32_t B, tn_ctx *const *ctxs, double *E, uint64_t *limb
     return wa > wb;
   });
   const CountRep rep = count_rep(3);   // the range of 3 61-bit primes + witness
-  const int P = limbs ? rep.P : 0;
+  const int P = limbs ? rep.P : 0;     // planes of a group at most
   size_t stage_bytes = 0;
   for (auto &ids : groups) stage_bytes += ids.size() * (4 + 8 * (size_t)P) + 64;
   char *stage = nullptr;
@@ -1280,6 +1389,8 @@ tn_status tn_batch_run(int32_t B, tn_ctx *const *ctxs, double *E, uint64_t *limb
     Program *p = nullptr;
     char *raw = nullptr;
     uint64_t *res = nullptr;
+    bool sat = false;
+    std::vector<float> J, h;   // the group's couplings
     tn_status s = TN_OK;
   };
   std::vector<Run> runs(groups.size());
@@ -1299,7 +1410,10 @@ tn_status tn_batch_run(int32_t B, tn_ctx *const *ctxs, double *E, uint64_t *limb
     off += (size_t)G * 8 * P;
     r.raw = stage + off;
     off += ((size_t)G * 4 + 63) / 64 * 64;
-    std::vector<float> J((size_t)G * n.m), h(n.h.empty() ? 0 : (size_t)G * n.n);
+    r.sat = limbs && sat_first(r.owner);
+    std::vector<float> &J = r.J, &h = r.h;
+    J.resize((size_t)G * n.m);
+    h.resize(n.h.empty() ? 0 : (size_t)G * n.n);
     for (int g = 0; g < G; ++g) {
       const Net &ng = ctxs[ids[g]]->net;
       std::copy(ng.J.begin(), ng.J.end(), J.begin() + (size_t)g * n.m);
@@ -1318,9 +1432,10 @@ tn_status tn_batch_run(int32_t B, tn_ctx *const *ctxs, double *E, uint64_t *limb
     r.owner->stream = st;
     RunArgs ra;
     r.s = batch_setup(r.owner, G, J.data(), h.empty() ? nullptr : h.data(), 0,
-                      limbs ? PM_COUNT : PM_ENERGY, P, &r.p, &ra, rep.rb);
+                      limbs ? PM_COUNT : PM_ENERGY, r.sat ? 1 : P, &r.p, &ra,
+                      r.sat ? 8 : rep.rb, r.sat);
     if (r.s == TN_OK) r.s = run_program(r.owner, *r.p, 0, -1, ra);
-    if (r.s == TN_OK) r.s = stage_results(r.owner, *r.p, G, P, r.raw, r.res);
+    if (r.s == TN_OK) r.s = stage_results(r.owner, *r.p, G, r.sat ? 1 : P, r.raw, r.res);
   }
   for (size_t gi = 0; gi < groups.size(); ++gi) {
     const std::vector<int> &ids = groups[gi];
@@ -1338,7 +1453,16 @@ tn_status tn_batch_run(int32_t B, tn_ctx *const *ctxs, double *E, uint64_t *limb
     tn_status s = r.s;
     if (s == TN_OK && limbs) {
       std::vector<uint64_t> lg((size_t)G * limbs_per);
-      s = finish_counts(r.owner, G, rep, r.raw, r.res, lg.data(), limbs_per, Eg.data(), sg.data());
+      s = finish_counts(r.owner, G, rep, r.raw, r.res, lg.data(), limbs_per, Eg.data(), sg.data(),
+                        r.sat);
+      std::vector<int> over;
+      for (int g = 0; r.sat && g < G; ++g)
+        if (r.res[g] == kSaturated) over.push_back(g);
+      if (!over.empty()) {
+        count_residues(r.owner, over, r.J.data(), r.h.empty() ? nullptr : r.h.data(), 0, rep,
+                       lg.data(), limbs_per, Eg.data(), sg.data());
+        s = first_of(sg.data(), G);
+      }
       for (int g = 0; g < G; ++g)
         std::copy(lg.begin() + (size_t)g * limbs_per, lg.begin() + (size_t)(g + 1) * limbs_per,
                   limbs + (int64_t)ids[g] * limbs_per);
@@ -1418,7 +1542,9 @@ tn_status tn_plan_info(const tn_ctx *ctx, int32_t *n_steps, int32_t *n_transpose
   }
   if (arena_count) {
     const CountRep rep = count_rep(3);
-    if (!build_program(ctx->net, ctx->plan, PM_COUNT, ctx->dt, rep.P, 0, &pn, &err, rep.rb))
+    const bool sat = sat_first(ctx);
+    if (!build_program(ctx->net, ctx->plan, PM_COUNT, ctx->dt, sat ? 1 : rep.P, 0, &pn, &err,
+                       sat ? 8 : rep.rb, sat))
       return TN_EINVAL;
     *arena_count = pn.arena_bytes;
   }
@@ -1434,6 +1560,11 @@ tn_status tn_plan_launches(const tn_ctx *ctx, int32_t mode, int64_t *counts) {
   const CountRep rep = count_rep(3);
   if (!build_program(ctx->net, ctx->plan, pm, ctx->dt, pm == PM_COUNT ? rep.P : 0, 0, &pg, &err,
                      pm == PM_COUNT ? rep.rb : 8))
+    return TN_EINVAL;
+  // counts run with one plane of exact integers first where they are likely to fit
+  // (the residue program above is then the one that saturated counts run on)
+  if (pm == PM_COUNT && sat_first(ctx) &&
+      !build_program(ctx->net, ctx->plan, pm, ctx->dt, 1, 0, &pg, &err, 8, true))
     return TN_EINVAL;
   for (int k = 0; k < 7; ++k) counts[k] = 0;
   for (const Op &op : pg.ops) {
@@ -1629,6 +1760,7 @@ void tn_destroy(tn_ctx *ctx) {
   if (!ctx) return;
   for (auto &p : ctx->prog) if (p) free_program(p.get());
   if (ctx->prog_pass) free_program(ctx->prog_pass.get());
+  if (ctx->prog_sat) free_program(ctx->prog_sat.get());
   if (ctx->dev_ready) {
     cudaFree(ctx->d_J);
     cudaFree(ctx->d_h);

@@ -75,4 +75,25 @@ __device__ __forceinline__ void build_tables(const ChainParams &p, const T *X, T
   }
 }
 
+// digits of the fixed legs (bits of the outer index tau) -> table slice offset
+// (8 values per slice)
+__device__ __forceinline__ int tc_slice(const int4 &d, int64_t tau) {
+  const int s0 = d.z & 0xff, s1 = (d.z >> 8) & 0xff, s2 = (d.z >> 16) & 0xff;
+  const int f = (int)((tau >> s0) & 1) | ((int)((tau >> s1) & 1) << 1) |
+                ((int)((tau >> s2) & 1) << 2);
+  return d.y + f * 8;
+}
+
+// element offset of outer index tau in a layout whose segment shifts are ssh
+template <typename I>
+__device__ __forceinline__ I rc_base_l(const ChainParams &p, int64_t tau, const int32_t *ssh) {
+  I base = 0;
+  I t = (I)tau;
+  for (int sg = p.nseg - 1; sg >= 0; --sg) {
+    base += (t & (I)(p.seg_size[sg] - 1)) << ssh[sg];
+    t >>= p.seg_sh[sg];
+  }
+  return base;
+}
+
 }  // namespace tn

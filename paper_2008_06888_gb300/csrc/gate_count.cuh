@@ -19,13 +19,19 @@ namespace tn {
 // indices per thread; every value and residue of A (and of B, unless its counts
 // are all 1) is loaded before any is compared, then the counts of the maximal
 // k add up (ties) with predicated modular products.
-// Four consecutive 4-byte words (16-byte aligned) stored with one access.
+// Four consecutive words (16-byte aligned) stored with one or two 16-byte accesses.
 template <typename W>
 __device__ __forceinline__ void gtc_store4(W *dst, const W *src) {
   static_assert(sizeof(W) == 4, "4-byte words");
   *reinterpret_cast<uint4 *>(dst) =
       make_uint4(__builtin_bit_cast(uint32_t, src[0]), __builtin_bit_cast(uint32_t, src[1]),
                  __builtin_bit_cast(uint32_t, src[2]), __builtin_bit_cast(uint32_t, src[3]));
+}
+
+__device__ __forceinline__ void gtc_store4(Sat64 *dst, const Sat64 *src) {
+  ulonglong2 *d = reinterpret_cast<ulonglong2 *>(dst);
+  d[0] = make_ulonglong2(src[0].v, src[1].v);
+  d[1] = make_ulonglong2(src[2].v, src[3].v);
 }
 
 // VC: the NS outputs of an outer index are NS consecutive words of C (and of
@@ -156,27 +162,33 @@ bool launch_gate_tc_r(const GateParams &p, const T *A, const T *B, T *C, const R
     k_gate_tc<T, KS_, NS_, P_, R><<<blocks, 256, 0, st>>>(p, A, B, C, nA, nB, nC, ps, ib);   \
     return true;                                                                            \
   }
+// the forms with the plane count of the residue type: 7 or 1 of 4 bytes, 1 of
+// saturating counts
 #define TN_GTC_P(P_)                                                                          \
   TN_GTC(1, 1, P_) TN_GTC(1, 2, P_) TN_GTC(2, 1, P_) TN_GTC(1, 4, P_) TN_GTC(2, 4, P_)        \
   TN_GTC(2, 16, P_)
-  if (vc && p.Ks == 2 && p.Ns == 16 && (p.P == 7 || p.P == 1)) {
-    if (p.P == 7)
+  if constexpr (sizeof(R) == 4) {
+    if (vc && p.Ks == 2 && p.Ns == 16 && p.P == 7) {
       k_gate_tc<T, 2, 16, 7, R, true><<<blocks, 256, 0, st>>>(p, A, B, C, nA, nB, nC, ps, ib);
-    else
-      k_gate_tc<T, 2, 16, 1, R, true><<<blocks, 256, 0, st>>>(p, A, B, C, nA, nB, nC, ps, ib);
+      return true;
+    }
+    TN_GTC_P(7)
+  }
+  if (vc && p.Ks == 2 && p.Ns == 16 && p.P == 1) {
+    k_gate_tc<T, 2, 16, 1, R, true><<<blocks, 256, 0, st>>>(p, A, B, C, nA, nB, nC, ps, ib);
     return true;
   }
   TN_GTC_P(1)
-  TN_GTC_P(7)
 #undef TN_GTC_P
 #undef TN_GTC
   return false;
 }
 
-// launch the form of `p` with 4-byte planes; false when there is none
+// launch the form of `p` with 4-byte planes or one plane of saturating counts;
+// false when there is none
 template <typename T>
-bool launch_gate_tc_typed(const GateParams &p, const T *A, const T *B, T *C, const uint32_t *nA,
-                          const uint32_t *nB, uint32_t *nC, const PrimeSet &ps, const Batch &bt,
+bool launch_gate_tc_typed(const GateParams &p, const T *A, const T *B, T *C, const void *nA,
+                          const void *nB, void *nC, const PrimeSet &ps, const Batch &bt,
                           cudaStream_t st) {
   int64_t nb = ((p.outer + 1) / 2 + 255) / 256;
   const int64_t cap = (int64_t)num_sms() * 32;
@@ -190,8 +202,12 @@ bool launch_gate_tc_typed(const GateParams &p, const T *A, const T *B, T *C, con
             (uint64_t)bt.ib % 16 == 0 && p.planeC % 4 == 0;
   for (int n = 0; vc && n < p.Ns; ++n) vc = p.nC[n] == n;
   for (int s = 0; vc && s < p.nseg; ++s) vc = p.seg_sC[s] % 4 == 0;
-  return launch_gate_tc_r<T, uint32_t>(p, A, B, C, nA, nB, nC, ps, dim3((unsigned)nb, bt.B), bt.ib,
-                                       vc, st);
+  const dim3 grid((unsigned)nb, bt.B);
+  if (ps.r32)
+    return launch_gate_tc_r<T, uint32_t>(p, A, B, C, (const uint32_t *)nA, (const uint32_t *)nB,
+                                         (uint32_t *)nC, ps, grid, bt.ib, vc, st);
+  return launch_gate_tc_r<T, Sat64>(p, A, B, C, (const Sat64 *)nA, (const Sat64 *)nB,
+                                    (Sat64 *)nC, ps, grid, bt.ib, vc, st);
 }
 
 }  // namespace tn

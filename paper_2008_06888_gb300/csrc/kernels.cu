@@ -78,7 +78,7 @@ static int64_t resident_slots(K kernel, int threads, size_t smem) {
 // instance, B instances and `slots` resident blocks: whole waves when a
 // multiple of the slots is within 16 waves, else about 8 waves so the last,
 // partial one is a small part of the launch.
-static int64_t wave_blocks(int64_t need, int B, int64_t slots) {
+int64_t wave_blocks(int64_t need, int B, int64_t slots) {
   if (need * B <= slots) return need;
   const int64_t whole = slots / std::gcd(slots, (int64_t)B);
   if (whole <= need && whole * B <= 16 * slots) return whole;
@@ -458,12 +458,19 @@ __device__ __forceinline__ void ld4(const uint32_t *p, uint32_t *o) {
   const uint4 a = *reinterpret_cast<const uint4 *>(p);
   o[0] = a.x; o[1] = a.y; o[2] = a.z; o[3] = a.w;
 }
+__device__ __forceinline__ void ld4(const Sat64 *p, Sat64 *o) {
+  ld4(reinterpret_cast<const uint64_t *>(p), reinterpret_cast<uint64_t *>(o));
+}
 __device__ __forceinline__ void st4(uint64_t *p, const uint64_t *v) {
   *reinterpret_cast<ulonglong2 *>(p) = make_ulonglong2(v[0], v[1]);
   *reinterpret_cast<ulonglong2 *>(p + 2) = make_ulonglong2(v[2], v[3]);
 }
 __device__ __forceinline__ void st4(uint32_t *p, const uint32_t *v) {
   *reinterpret_cast<uint4 *>(p) = make_uint4(v[0], v[1], v[2], v[3]);
+}
+
+__device__ __forceinline__ void st4(Sat64 *p, const Sat64 *v) {
+  st4(reinterpret_cast<uint64_t *>(p), reinterpret_cast<const uint64_t *>(v));
 }
 
 template <typename T, int KS, int NS, int P, typename R = uint64_t>
@@ -597,8 +604,9 @@ template <typename T>
 static bool launch_gate2c(const GateParams &p, const T *A, const T *B, T *C, const uint64_t *nA,
                           const uint64_t *nB, uint64_t *nC, const PrimeSet &ps, const Batch &bt,
                           cudaStream_t st) {
-  // 4 planes of 8-byte residues or 7 of 4-byte ones
-  if (!((p.P == 4 && !ps.r32) || (p.P == 7 && ps.r32)) || std::getenv("TN_NO_GATE2")) return false;
+  // 4 planes of 8-byte residues, 7 of 4-byte ones, or one of saturating counts
+  if (!(((p.P == 4 || p.P == 1) && !ps.r32) || (p.P == 7 && ps.r32)) || std::getenv("TN_NO_GATE2"))
+    return false;
   GateParams q = p;
   q.P = 0;   // gate2_form checks the value layout; the planes share it
   Gate2 g;
@@ -623,6 +631,11 @@ static bool launch_gate2c(const GateParams &p, const T *A, const T *B, T *C, con
     TN_G2C(1, 2, 7, uint32_t)
     TN_G2C(2, 1, 7, uint32_t)
     TN_G2C(2, 2, 7, uint32_t)
+  } else if (p.P == 1) {
+    TN_G2C(1, 1, 1, Sat64)
+    TN_G2C(1, 2, 1, Sat64)
+    TN_G2C(2, 1, 1, Sat64)
+    TN_G2C(2, 2, 1, Sat64)
   } else {
     TN_G2C(1, 1, 4, uint64_t)
     TN_G2C(1, 2, 4, uint64_t)
@@ -682,11 +695,9 @@ cudaError_t launch_gate(Dtype dt, const GateParams &p, const void *xA, const voi
                      : launch_gate2c<int32_t>(p, (const int32_t *)xA, (const int32_t *)xB,
                                               (int32_t *)xC, nA, nB, nC, ps, bt, st);
     if (streamed) return cudaGetLastError();
-    if (ps.r32 && !std::getenv("TN_NO_GATE_TC")) {
-      const uint32_t *a = (const uint32_t *)nA, *b = (const uint32_t *)nB;
-      uint32_t *c = (uint32_t *)nC;
-      if (dt == DT_F32 ? launch_gate_tc_f32(p, xA, xB, xC, a, b, c, ps, bt, st)
-                       : launch_gate_tc_i32(p, xA, xB, xC, a, b, c, ps, bt, st))
+    if ((ps.r32 || p.P == 1) && !std::getenv("TN_NO_GATE_TC")) {
+      if (dt == DT_F32 ? launch_gate_tc_f32(p, xA, xB, xC, nA, nB, nC, ps, bt, st)
+                       : launch_gate_tc_i32(p, xA, xB, xC, nA, nB, nC, ps, bt, st))
         return cudaGetLastError();
     }
   }
@@ -1110,7 +1121,7 @@ __device__ __forceinline__ void cas_addmod(uint64_t *dst, uint64_t v, uint64_t c
   unsigned long long old = *d, assumed;
   do {
     assumed = old;
-    old = atomicCAS(d, assumed, (unsigned long long)addmod61(assumed, v, c));
+    old = atomicCAS(d, assumed, (unsigned long long)addmodR((uint64_t)assumed, v, c));
   } while (old != assumed);
 }
 __device__ __forceinline__ void cas_addmod(uint32_t *dst, uint32_t v, uint64_t c) {
@@ -1435,6 +1446,11 @@ cudaError_t launch_gemm_count(Dtype dt, const GemmParams &p, const void *xA, con
     if (ps.r32 && p.P == 1) {
       if (f) launch_gemm_count_t<float, uint32_t, 1>(p, xA, xB, xC, nA, nB, nC, ps, bt, st);
       else launch_gemm_count_t<int32_t, uint32_t, 1>(p, xA, xB, xC, nA, nB, nC, ps, bt, st);
+      return cudaGetLastError();
+    }
+    if (!ps.r32 && p.P == 1) {
+      if (f) launch_gemm_count_t<float, Sat64, 1>(p, xA, xB, xC, nA, nB, nC, ps, bt, st);
+      else launch_gemm_count_t<int32_t, Sat64, 1>(p, xA, xB, xC, nA, nB, nC, ps, bt, st);
       return cudaGetLastError();
     }
     if (!ps.r32 && p.P == 4) {
@@ -1847,6 +1863,8 @@ cudaError_t launch_chain(Dtype dt, const ChainParams &p, const char *arena, cons
                          const uint64_t *An, void *Cx, uint64_t *Cn, const PrimeSet &ps,
                          const Batch &bt, cudaStream_t st) {
   if (p.outer == 0) return cudaSuccess;
+  if (p.mode == 1 && p.P == 1 && p.ntg > 0)
+    return launch_schain(p, arena, Ax, An, Cx, Cn, bt, st);
   if (p.mode == 1 && p.P > 0) return launch_rchain_count(dt, p, arena, Ax, An, Cx, Cn, ps, bt, st);
   if (p.mode == 1) return launch_rchain(dt, p, arena, Ax, Cx, bt, st);
   const bool c = p.P > 0;
@@ -2235,27 +2253,6 @@ __device__ __forceinline__ void tc_contract(int code, T (&v)[1 << RB], const V &
 #undef TC_C
 }
 
-// digits of the fixed legs (bits of the outer index tau) -> table slice offset
-// (8 values per slice)
-__device__ __forceinline__ int tc_slice(const int4 &d, int64_t tau) {
-  const int s0 = d.z & 0xff, s1 = (d.z >> 8) & 0xff, s2 = (d.z >> 16) & 0xff;
-  const int f = (int)((tau >> s0) & 1) | ((int)((tau >> s1) & 1) << 1) |
-                ((int)((tau >> s2) & 1) << 2);
-  return d.y + f * 8;
-}
-
-// element offset of outer index tau in a layout whose segment shifts are ssh
-template <typename I>
-__device__ __forceinline__ I rc_base_l(const ChainParams &p, int64_t tau, const int32_t *ssh) {
-  I base = 0;
-  I t = (I)tau;
-  for (int sg = p.nseg - 1; sg >= 0; --sg) {
-    base += (t & (I)(p.seg_size[sg] - 1)) << ssh[sg];
-    t >>= p.seg_sh[sg];
-  }
-  return base;
-}
-
 // The register-chain pipeline of k_rchain with table gates: the descriptor of
 // gate gi+2 and the table slice of gate gi+1 are loaded while gate gi runs.
 template <typename T, int RB, typename I, int STAGES, int MINB, int NT = 256>
@@ -2596,7 +2593,8 @@ static int low_legs_first(const ChainParams &p, ChainParams *q) {
 cudaError_t launch_rchain_count(Dtype dt, const ChainParams &p, const char *arena,
                                 const void *Ax, const uint64_t *An, void *Cx, uint64_t *Cn,
                                 const PrimeSet &ps, const Batch &bt, cudaStream_t st) {
-  if (p.t != 3 || !((p.P == 4 && !ps.r32) || (p.P == 7 && ps.r32))) return cudaErrorInvalidValue;
+  if (p.t != 3 || !(((p.P == 4 || p.P == 1) && !ps.r32) || (p.P == 7 && ps.r32)))
+    return cudaErrorInvalidValue;
   const int64_t need = (p.outer + 255) / 256;
   // vector accesses (4-byte residues): the low legs lead, and every array
   // start, plane distance and instance stride is a multiple of the vector
@@ -2622,11 +2620,13 @@ cudaError_t launch_rchain_count(Dtype dt, const ChainParams &p, const char *aren
         reinterpret_cast<R_ *>(Cn), ps, bt.ib);                                                  \
   } while (0)
   if (dt == DT_F32) {
-    if (!ps.r32) TN_RCC(float, 4, uint64_t, 0);
+    if (p.P == 1) TN_RCC(float, 1, Sat64, 0);
+    else if (!ps.r32) TN_RCC(float, 4, uint64_t, 0);
     else if (lw == 2) TN_RCC(float, 7, uint32_t, 2);
     else if (lw == 1) TN_RCC(float, 7, uint32_t, 1);
     else TN_RCC(float, 7, uint32_t, 0);
   } else {
+    if (p.P == 1) return cudaErrorInvalidValue;   // integral contexts run k_schain
     if (!ps.r32) TN_RCC(int32_t, 4, uint64_t, 0);
     else if (lw == 2) TN_RCC(int32_t, 7, uint32_t, 2);
     else if (lw == 1) TN_RCC(int32_t, 7, uint32_t, 1);

@@ -33,13 +33,13 @@ cudaError_t launch_gate(Dtype dt, const GateParams &p, const void *xA, const voi
                         const Batch &bt, cudaStream_t st);
 
 // Counting gate contraction with compile-time (K, N, planes) forms for 4-byte
-// residue planes (gate_count_*.cu); false when the step has no such form (the
-// generic kernel runs it).
+// residue planes and for one plane of saturating 64-bit counts (gate_count_*.cu);
+// false when the step has no such form (the generic kernel runs it).
 bool launch_gate_tc_i32(const GateParams &p, const void *A, const void *B, void *C,
-                        const uint32_t *nA, const uint32_t *nB, uint32_t *nC, const PrimeSet &ps,
+                        const void *nA, const void *nB, void *nC, const PrimeSet &ps,
                         const Batch &bt, cudaStream_t st);
 bool launch_gate_tc_f32(const GateParams &p, const void *A, const void *B, void *C,
-                        const uint32_t *nA, const uint32_t *nB, uint32_t *nC, const PrimeSet &ps,
+                        const void *nA, const void *nB, void *nC, const PrimeSet &ps,
                         const Batch &bt, cudaStream_t st);
 
 // Register-tiled max-plus GEMM (128 x 128 tiles, cp.async staging), values only.
@@ -74,6 +74,16 @@ cudaError_t launch_chain(Dtype dt, const ChainParams &p, const char *arena, cons
                          const uint64_t *An, void *Cx, uint64_t *Cn, const PrimeSet &ps,
                          const Batch &bt, cudaStream_t st);
 size_t chain_smem_bytes(const ChainParams &p, size_t elem);
+
+// Folded register chain of INT32 values with one plane of saturating 64-bit
+// counts (chain_sat.cu).
+cudaError_t launch_schain(const ChainParams &p, const char *arena, const void *Ax,
+                          const uint64_t *An, void *Cx, uint64_t *Cn, const Batch &bt,
+                          cudaStream_t st);
+
+// Resident blocks of a kernel on the whole device and the grid (blocks per
+// instance) of a grid-stride kernel with `need` blocks of work per instance.
+int64_t wave_blocks(int64_t need, int B, int64_t slots);
 
 // dE/dJ and dE/dh at the traced state.
 cudaError_t launch_grad(int q, int n, int m, const int32_t *eu, const int32_t *ev,

@@ -1,6 +1,7 @@
 // modarith.cuh -- modular arithmetic of the counting residue planes (device):
 // 61-bit primes 2^61 - c in 8-byte residues and 31-bit primes 2^31 - c in
-// 4-byte ones, c < 2^10, reduced after Crandall's pseudo-Mersenne method.
+// 4-byte ones, c < 2^10, reduced after Crandall's pseudo-Mersenne method; and the
+// saturating 64-bit counts of the exact single-plane programs.
 #pragma once
 #include <stdint.h>
 
@@ -46,15 +47,40 @@ __device__ __forceinline__ uint32_t addmod31(uint32_t a, uint32_t b, uint64_t c)
   const uint32_t s = a + b;                            // < 2p < 2^32
   return s >= p ? s - p : s;
 }
-// residue arithmetic by plane width
+// Exact counts below 2^64 - 1 in one 8-byte plane, saturating: min(n, 2^64 - 1)
+// is compatible with sums and products of counts (which are never negative), so
+// a result below the cap is exact whatever its intermediates did, and one at the
+// cap says that the count needs the residue planes.
+__device__ __forceinline__ uint64_t addsat64(uint64_t a, uint64_t b) {
+  const uint64_t s = a + b;
+  return s < a ? ~0ull : s;
+}
+__device__ __forceinline__ uint64_t mulsat64(uint64_t a, uint64_t b) {
+  return __umul64hi(a, b) ? ~0ull : a * b;
+}
+// A saturating count as a type of its own: the hot kernels' forms carry no
+// modular code.
+struct Sat64 {
+  uint64_t v;
+  Sat64() = default;
+  __device__ __forceinline__ Sat64(int x) : v((uint64_t)x) {}
+  __device__ __forceinline__ explicit Sat64(uint64_t x) : v(x) {}
+};
+__device__ __forceinline__ Sat64 mulmodR(Sat64 a, Sat64 b, uint64_t) {
+  return Sat64(mulsat64(a.v, b.v));
+}
+__device__ __forceinline__ Sat64 addmodR(Sat64 a, Sat64 b, uint64_t) {
+  return Sat64(addsat64(a.v, b.v));
+}
+// residue arithmetic by plane width; c == 0 in an 8-byte plane: saturating counts
 __device__ __forceinline__ uint64_t mulmodR(uint64_t a, uint64_t b, uint64_t c) {
-  return mulmod61(a, b, c);
+  return c == 0 ? mulsat64(a, b) : mulmod61(a, b, c);
 }
 __device__ __forceinline__ uint32_t mulmodR(uint32_t a, uint32_t b, uint64_t c) {
   return mulmod31(a, b, c);
 }
 __device__ __forceinline__ uint64_t addmodR(uint64_t a, uint64_t b, uint64_t c) {
-  return addmod61(a, b, c);
+  return c == 0 ? addsat64(a, b) : addmod61(a, b, c);
 }
 __device__ __forceinline__ uint32_t addmodR(uint32_t a, uint32_t b, uint64_t c) {
   return addmod31(a, b, c);

@@ -653,7 +653,11 @@ struct Builder {
   }
 
   // Rank-changing steps at the ends of a folded register chain (values, q = 2).
-  bool rank_fusion() const { return regmode && fold && P == 0 && kRB >= 5; }
+  bool rank_fusion() const { return regmode && folded() && kRB >= (P == 0 ? 5 : 4); }
+  // whether register chains run on folded table gates: value programs, and exact
+  // 64-bit counts of integral values (sums of any order tie alike there; float
+  // counts keep the unfolded order of additions, on which their ties depend)
+  bool folded() const { return fold && (P == 0 || (pr.sat && pr.dt == DT_I32)); }
 
   // a step adding one leg to `big` (no contraction, one batch leg at most): the
   // chain starts from big, the new leg slowest (or innermost with
@@ -869,7 +873,7 @@ struct Builder {
       blocs->push_back(loc[g.btensor]);
     }
     cp.P = P;
-    if (P == 0 && fold) fold_reg_chain(cp);
+    if (folded()) fold_reg_chain(cp);
     return cp;
   }
 
@@ -1155,7 +1159,7 @@ struct Builder {
   bool build(ProgMode mode, int64_t seg_bytes) {
     fuse = std::getenv("TN_NO_FUSION") == nullptr;
     // register chains: q = 2 values, or q = 2 counts with 3 primes + witness
-    regmode = q == 2 && (P == 0 || (P == 4 && rb == 8) || (P == 7 && rb == 4)) &&
+    regmode = q == 2 && (P == 0 || (P == 4 && rb == 8) || (P == 7 && rb == 4) || pr.sat) &&
               std::getenv("TN_TILE_CHAINS") == nullptr;
     fold = std::getenv("TN_NO_FOLD") == nullptr;
     grow_inner = std::getenv("TN_GROW_INNER") != nullptr;
@@ -1164,6 +1168,10 @@ struct Builder {
     kRB = fold ? 6 : 5;
     if (const char *rb = std::getenv("TN_REG_BITS")) kRB = std::max(4, std::min(fold ? 6 : 5, std::atoi(rb)));
     if (P > 0) kRB = 3;
+    // exact 64-bit counts: 12 bytes per state, 2^5 states per thread
+    if (pr.sat && folded()) kRB = std::getenv("TN_SAT_RB") ? std::atoi(std::getenv("TN_SAT_RB")) : 5;
+    // integral counts without folding have no register-chain kernel
+    if (pr.sat && !folded() && pr.dt == DT_I32) regmode = false;
     if (q == 3) { tmax = 7; wlow = 4; }
     emit_leaves();
     if (!forward()) return false;
@@ -1233,7 +1241,7 @@ void plan_memory(Program &pr) {
 int64_t abs_off(const Program &pr, const Loc &l) { return pr.bufs[l.buf].off + l.xoff; }
 
 bool build_program(const Net &net, const Plan &plan, ProgMode mode, Dtype dt, int P,
-                   int64_t seg_bytes, Program *pr, std::string *err, int rbytes) {
+                   int64_t seg_bytes, Program *pr, std::string *err, int rbytes, bool sat) {
   *pr = Program();
   pr->mode = mode;
   pr->dt = dt;
@@ -1243,7 +1251,12 @@ bool build_program(const Net &net, const Plan &plan, ProgMode mode, Dtype dt, in
     *err = "residue width must be 4 or 8 bytes";
     return false;
   }
+  if (sat && (mode != PM_COUNT || P != 1 || rbytes != 8)) {
+    *err = "saturating counts need a counting program with one 8-byte plane";
+    return false;
+  }
   pr->rbytes = rbytes;
+  pr->sat = sat;
   Builder bd(net, plan, *pr);
   if (!bd.build(mode, seg_bytes)) {
     *err = bd.err.empty() ? "program: lowering failed" : bd.err;

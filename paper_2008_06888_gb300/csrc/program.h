@@ -42,6 +42,7 @@ struct Program {
   int q = 2, P = 0;
   int rbytes = 8;                    // bytes of one residue of the counting planes
   bool pass_prime = false;           // one 31-bit prime per pass: plane 0's prime is set per run
+  bool sat = false;                  // one 8-byte plane of exact, saturating 64-bit counts
   std::vector<BufInfo> bufs;
   std::vector<Op> ops;
   std::vector<GateParams> gates;
@@ -82,9 +83,11 @@ struct Program {
 // Build the program for a plan.  seg_bytes: traceback checkpoint segment
 // budget (PM_CONFIG; <= 0 keeps every intermediate).
 // rbytes: bytes of one residue of the counting planes (8: 61-bit primes; 4:
-// 31-bit primes, the one-prime-per-pass counts).
+// 31-bit primes, the one-prime-per-pass counts).  sat (PM_COUNT, P = 1, rbytes
+// = 8): the plane holds exact counts that saturate at 2^64 - 1.
 bool build_program(const Net &net, const Plan &plan, ProgMode mode, Dtype dt, int P,
-                   int64_t seg_bytes, Program *pr, std::string *err, int rbytes = 8);
+                   int64_t seg_bytes, Program *pr, std::string *err, int rbytes = 8,
+                   bool sat = false);
 
 int64_t abs_off(const Program &pr, const Loc &l);  // arena byte offset of values
 

@@ -200,6 +200,7 @@ struct ChainTrace {
 
 // 61-bit pseudo-Mersenne primes p = 2^61 - c (reduction after Crandall), or,
 // for counts run one prime per pass in 4-byte planes, 31-bit ones 2^31 - c.
+// c == 0 with 8-byte planes: no modulus, the plane holds saturating 64-bit counts.
 struct PrimeSet {
   uint64_t c[TN_MAX_PRIMES];
   int32_t r32;   // 1: residue planes hold uint32 residues of primes 2^31 - c

@@ -658,20 +658,22 @@ CountRep count_rep(int n_primes) {
   return r;
 }
 
-// Counts below 2^64 - 1 need no residues: one 8-byte plane holds them exactly,
+// Counts below 2^59 need no residues: one 8-byte plane holds them exactly,
 // 4 + 8 bytes per element instead of 4 + 28 (mixed +-J batches of side 8..20: 192
 // instances in @@ ms instead of 46.6), and saturates where they do not fit; such an
 // instance is run again with the residue planes.  Contexts whose counts are likely to
 // be larger start there: +-J glasses have up to about 0.105 bits of ground-state
 // entropy per spin without fields (square lattices; 3-regular and chimera graphs less),
-// Max-2-SAT formulas about 0.35 bits per variable, so 64 bits hold up to some 600 spins
-// without and 180 with fields.  TN_COUNT_RESIDUES keeps the residue planes.
+// Max-2-SAT formulas about 0.35 bits per variable, so 59 bits hold up to some 540 spins
+// without and 165 with fields.  TN_COUNT_RESIDUES keeps the residue planes.
 bool sat_first(const tn_ctx *ctx) {
   for (const char *v : {"TN_COUNT_RESIDUES", "TN_COUNT_61", "TN_COUNT_PASSES"})
     if (std::getenv(v)) return false;
-  return ctx->net.n <= (ctx->net.h.empty() ? 600 : 180) || ctx->dt == DT_F32;
+  return ctx->net.n <= (ctx->net.h.empty() ? 540 : 165) || ctx->dt == DT_F32;
 }
-constexpr uint64_t kSaturated = ~0ull;
+// an exact count stays below this; one at or above it may have saturated (the chain
+// kernel's cap, chain_sat.cu)
+constexpr uint64_t kSaturated = 1ull << 59;
 
 // exact count from residues res[i] modulo rep.primes[i] (the last one the witness)
 tn_status count_from_residues(tn_ctx *ctx, const std::vector<uint64_t> &res, const CountRep &rep,
@@ -1007,7 +1009,7 @@ tn_status tn_count(tn_ctx *ctx, int32_t n_primes, uint64_t *limbs, int32_t *n_li
       CK(cudaMemcpyAsync(raw, base + p->root.xoff, 4, cudaMemcpyDeviceToHost, ctx->stream));
       CK(cudaMemcpyAsync(&v, base + p->root.noff, 8, cudaMemcpyDeviceToHost, ctx->stream));
       CK(cudaStreamSynchronize(ctx->stream));
-      if (v != kSaturated) {
+      if (v < kSaturated) {
         if (E) *E = root_energy(ctx, raw);
         return finish_count(ctx, residues_of(v, rep), rep.primes, limbs, n_limbs, ln_count);
       }
@@ -1196,7 +1198,7 @@ tn_status finish_counts(tn_ctx *ctx, int B, const CountRep &rep, const char *raw
   const int P = rep.P;
   tn_status first = TN_OK;
   for (int b = 0; b < B; ++b) {
-    if (sat && res[b] == kSaturated) continue;
+    if (sat && res[b] >= kSaturated) continue;
     if (E) E[b] = root_energy(ctx, raw + 4 * b);
     std::vector<uint64_t> r(P), v;
     if (sat) r = residues_of(res[b], rep);
@@ -1296,7 +1298,7 @@ tn_status tn_count_batch(tn_ctx *ctx, int32_t B, const float *J, const float *h,
   s = finish_counts(ctx, B, rep, raw.data(), res.data(), limbs, limbs_per, E, status, sat);
   std::vector<int> over;
   for (int b = 0; sat && b < B; ++b)
-    if (res[b] == kSaturated) over.push_back(b);
+    if (res[b] >= kSaturated) over.push_back(b);
   if (over.empty()) return s;
   s = count_residues(ctx, over, J, h, on_device, rep, limbs, limbs_per, E, status);
   return s != TN_OK ? s : first_of(status, B);
@@ -1457,7 +1459,7 @@ tn_status tn_batch_run(int32_t B, tn_ctx *const *ctxs, double *E, uint64_t *limb
                         r.sat);
       std::vector<int> over;
       for (int g = 0; r.sat && g < G; ++g)
-        if (r.res[g] == kSaturated) over.push_back(g);
+        if (r.res[g] >= kSaturated) over.push_back(g);
       if (!over.empty()) {
         count_residues(r.owner, over, r.J.data(), r.h.empty() ? nullptr : r.h.data(), 0, rep,
                        lg.data(), limbs_per, Eg.data(), sg.data());

@@ -2,12 +2,11 @@
 // values and one plane of saturating 64-bit counts (q = 2), folded table gates.
 //
 // A thread owns the 2^RB states of the chain's register legs for one outer index:
-// RB = 5 legs and 12 bytes per state fill about 96 registers, against 3 legs with
-// the seven 4-byte residue planes of the modular counts.  One pass then moves
-// (4 + 8) bytes per element each way for up to five replaced legs, where the
-// residue form moves (4 + 28) for three.  The bound is HBM; a replace gate costs
-// about 11 instructions per state (two sums, a maximum, two comparisons, the
-// selection of the 64-bit count, half of a saturating sum).
+// RB = 4 legs and 12 bytes per state are 48 registers, against 3 legs with the seven
+// 4-byte residue planes of the modular counts.  One pass then moves (4 + 8) bytes per
+// element each way for up to four replaced legs, where the residue form moves (4 + 28)
+// for three.  A replace gate costs about 10 instructions per state (two sums, a
+// maximum, two comparisons, the selection of the 64-bit count, half of its sum).
 //
 // Gate counts: a leaf operand counts 1 everywhere, so a table gate made of leaves
 // only selects and adds the states' counts; otherwise its count table (the product
@@ -77,57 +76,72 @@ __device__ __forceinline__ void sstore(uint64_t *dst, const uint64_t *src) {
   }
 }
 
+// Saturation inside a chain: the upper words of the counts are clamped when they are
+// loaded (to kCap + 2^32 at most) and after every fourth gate, and a gate at most
+// doubles a count, so sums never wrap.  Counts below kCap are exact; a sum or product
+// with a term of kCap or more is itself at least kCap.  (One instruction per clamp,
+// against five per saturating 64-bit sum.)
+constexpr uint32_t kCapHi = 1u << 27;   // kCap = 2^59
+__device__ __forceinline__ uint64_t clamp_count(uint64_t n) {
+  const uint32_t hi = min((uint32_t)(n >> 32), kCapHi);
+  return ((uint64_t)hi << 32) | (uint32_t)n;
+}
+__device__ __forceinline__ uint64_t mulcap(uint64_t a, uint64_t b) {
+  return clamp_count(mulsat64(a, b));
+}
+
 // (x, n) of the larger of two terms, counts added on a tie (both: their sum)
 __device__ __forceinline__ uint64_t tie(int32_t x, int32_t y, uint64_t nx, uint64_t ny,
                                         uint64_t both) {
   return x > y ? nx : (x < y ? ny : both);
 }
 
-// Replace (CON: final contraction, no new digit) on register bit J; km: bit of the
-// extra register leg (0: none) choosing between the table halves lo and hi, each
-// (x, x') = (0,0), (1,0), (0,1), (1,1).  cn: count table in the same order, null
-// when every count is 1.
-template <int RB, int J, bool CON>
+// Replace (CON: final contraction, no new digit) on register bit J with the extra
+// register leg K (-1: none), whose digit chooses between the table halves lo and hi,
+// each (x, x') = (0,0), (1,0), (0,1), (1,1).
+template <int RB, int J, int K, bool CON>
 __device__ __forceinline__ void srep(int32_t (&v)[1 << RB], uint64_t (&n)[1 << RB], const int4 &lo,
-                                     const int4 &hi, int km, const uint64_t *cn) {
-  if constexpr (J < RB) {
-    if (cn == nullptr) {
+                                     const int4 &hi) {
 #pragma unroll
-      for (int e = 0; e < (1 << RB); ++e) {
-        if (e & (1 << J)) continue;
-        const int e1 = e | (1 << J);
-        const bool k = (e & km) != 0;
-        const int32_t a = v[e], b = v[e1];
-        const uint64_t na = n[e], nb = n[e1], both = addsat64(na, nb);
-        const int32_t s00 = a + (k ? hi.x : lo.x), s10 = b + (k ? hi.y : lo.y);
-        v[e] = max(s00, s10);
-        n[e] = tie(s00, s10, na, nb, both);
-        if (!CON) {
-          const int32_t s01 = a + (k ? hi.z : lo.z), s11 = b + (k ? hi.w : lo.w);
-          v[e1] = max(s01, s11);
-          n[e1] = tie(s01, s11, na, nb, both);
-        }
-      }
-    } else {
+  for (int e = 0; e < (1 << RB); ++e) {
+    if (e & (1 << J)) continue;
+    const int e1 = e | (1 << J);
+    const bool k = K >= 0 && ((e >> (K < 0 ? 0 : K)) & 1);
+    const int32_t a = v[e], b = v[e1];
+    const uint64_t na = n[e], nb = n[e1], both = na + nb;
+    const int32_t s00 = a + (k ? hi.x : lo.x), s10 = b + (k ? hi.y : lo.y);
+    v[e] = max(s00, s10);
+    n[e] = tie(s00, s10, na, nb, both);
+    if (!CON) {
+      const int32_t s01 = a + (k ? hi.z : lo.z), s11 = b + (k ? hi.w : lo.w);
+      v[e1] = max(s01, s11);
+      n[e1] = tie(s01, s11, na, nb, both);
+    }
+  }
+}
+
+// The same with gate counts: cn is the count table in the order of lo, hi.
+template <int RB, int J, bool CON>
+__device__ __forceinline__ void srep_n(int32_t (&v)[1 << RB], uint64_t (&n)[1 << RB],
+                                       const int4 &lo, const int4 &hi, int km,
+                                       const uint64_t *cn) {
 #pragma unroll
-      for (int e = 0; e < (1 << RB); ++e) {
-        if (e & (1 << J)) continue;
-        const int e1 = e | (1 << J);
-        const bool k = (e & km) != 0;
-        const uint64_t *c = cn + (k ? 4 : 0);
-        const int32_t a = v[e], b = v[e1];
-        const uint64_t na = n[e], nb = n[e1];
-        const int32_t s00 = a + (k ? hi.x : lo.x), s10 = b + (k ? hi.y : lo.y);
-        const uint64_t p00 = mulsat64(na, c[0]), p10 = mulsat64(nb, c[1]);
-        v[e] = max(s00, s10);
-        n[e] = tie(s00, s10, p00, p10, addsat64(p00, p10));
-        if (!CON) {
-          const int32_t s01 = a + (k ? hi.z : lo.z), s11 = b + (k ? hi.w : lo.w);
-          const uint64_t p01 = mulsat64(na, c[2]), p11 = mulsat64(nb, c[3]);
-          v[e1] = max(s01, s11);
-          n[e1] = tie(s01, s11, p01, p11, addsat64(p01, p11));
-        }
-      }
+  for (int e = 0; e < (1 << RB); ++e) {
+    if (e & (1 << J)) continue;
+    const int e1 = e | (1 << J);
+    const bool k = (e & km) != 0;
+    const uint64_t *c = cn + (k ? 4 : 0);
+    const int32_t a = v[e], b = v[e1];
+    const uint64_t na = n[e], nb = n[e1];
+    const int32_t s00 = a + (k ? hi.x : lo.x), s10 = b + (k ? hi.y : lo.y);
+    const uint64_t p00 = mulcap(na, c[0]), p10 = mulcap(nb, c[1]);
+    v[e] = max(s00, s10);
+    n[e] = tie(s00, s10, p00, p10, p00 + p10);
+    if (!CON) {
+      const int32_t s01 = a + (k ? hi.z : lo.z), s11 = b + (k ? hi.w : lo.w);
+      const uint64_t p01 = mulcap(na, c[2]), p11 = mulcap(nb, c[3]);
+      v[e1] = max(s01, s11);
+      n[e1] = tie(s01, s11, p01, p11, p01 + p11);
     }
   }
 }
@@ -141,33 +155,45 @@ __device__ __forceinline__ void sdiag(int32_t (&v)[1 << RB], uint64_t (&n)[1 << 
   for (int e = 0; e < (1 << RB); ++e) {
     const bool x0 = (e & mj) != 0, x1 = (e & mk) != 0;
     v[e] = v[e] + (x1 ? (x0 ? lo.w : lo.z) : (x0 ? lo.y : lo.x));
-    if (cn != nullptr) n[e] = mulsat64(n[e], cn[(x0 ? 1 : 0) | (x1 ? 2 : 0)]);
+    if (cn != nullptr) n[e] = mulcap(n[e], cn[(x0 ? 1 : 0) | (x1 ? 2 : 0)]);
   }
 }
 
+// dispatch: replace on J with extra leg K is code J * 7 + K + 1, a contraction 100
+// above it; diagonal gates are 42 + (J + 1) * 7 + K + 1
 template <int RB>
 __device__ __forceinline__ void sapply(int code, int32_t (&v)[1 << RB], uint64_t (&n)[1 << RB],
                                        const int4 &lo, const int4 &hi, const uint64_t *cn) {
-  if (code >= 100) {
-    const int J = (code - 100) / 7, K = (code - 100) % 7 - 1, km = K >= 0 ? 1 << K : 0;
-    switch (J) {
-      case 0: srep<RB, 0, true>(v, n, lo, hi, km, cn); break;
-      case 1: srep<RB, 1, true>(v, n, lo, hi, km, cn); break;
-      case 2: srep<RB, 2, true>(v, n, lo, hi, km, cn); break;
-      case 3: srep<RB, 3, true>(v, n, lo, hi, km, cn); break;
-      default: srep<RB, 4, true>(v, n, lo, hi, km, cn); break;
+  static_assert(RB == 4, "the cases below are those of four register legs");
+  if (cn == nullptr) {
+#define TN_S(J, K)                                                     \
+  case (J) * 7 + (K) + 1: srep<RB, J, K, false>(v, n, lo, hi); break;    \
+  case 100 + (J) * 7 + (K) + 1: srep<RB, J, K, true>(v, n, lo, hi); break;
+    switch (code) {
+      TN_S(0, -1) TN_S(0, 1) TN_S(0, 2) TN_S(0, 3)
+      TN_S(1, -1) TN_S(1, 0) TN_S(1, 2) TN_S(1, 3)
+      TN_S(2, -1) TN_S(2, 0) TN_S(2, 1) TN_S(2, 3)
+      TN_S(3, -1) TN_S(3, 0) TN_S(3, 1) TN_S(3, 2)
+      default: sdiag<RB>(v, n, (code - 42) / 7 - 1, (code - 42) % 7 - 1, lo, cn); break;
     }
-  } else if (code >= 42) {
+#undef TN_S
+    return;
+  }
+  const bool con = code >= 100;
+  const int r = con ? code - 100 : code, J = r / 7, K = r % 7 - 1, km = K >= 0 ? 1 << K : 0;
+  if (!con && code >= 42) {
     sdiag<RB>(v, n, (code - 42) / 7 - 1, (code - 42) % 7 - 1, lo, cn);
-  } else {
-    const int J = code / 7, K = code % 7 - 1, km = K >= 0 ? 1 << K : 0;
-    switch (J) {
-      case 0: srep<RB, 0, false>(v, n, lo, hi, km, cn); break;
-      case 1: srep<RB, 1, false>(v, n, lo, hi, km, cn); break;
-      case 2: srep<RB, 2, false>(v, n, lo, hi, km, cn); break;
-      case 3: srep<RB, 3, false>(v, n, lo, hi, km, cn); break;
-      default: srep<RB, 4, false>(v, n, lo, hi, km, cn); break;
-    }
+    return;
+  }
+  switch (con ? J + 4 : J) {
+    case 0: srep_n<RB, 0, false>(v, n, lo, hi, km, cn); break;
+    case 1: srep_n<RB, 1, false>(v, n, lo, hi, km, cn); break;
+    case 2: srep_n<RB, 2, false>(v, n, lo, hi, km, cn); break;
+    case 3: srep_n<RB, 3, false>(v, n, lo, hi, km, cn); break;
+    case 4: srep_n<RB, 0, true>(v, n, lo, hi, km, cn); break;
+    case 5: srep_n<RB, 1, true>(v, n, lo, hi, km, cn); break;
+    case 6: srep_n<RB, 2, true>(v, n, lo, hi, km, cn); break;
+    default: srep_n<RB, 3, true>(v, n, lo, hi, km, cn); break;
   }
 }
 
@@ -245,6 +271,8 @@ __global__ void __launch_bounds__(NT, MINB) k_schain(const ChainParams p,
         sload<LWI>(src + o[e], &v[e]);
         sload<LWI>(srn + o[e], &n[e]);
       }
+#pragma unroll
+      for (int e = 0; e < (1 << RB); ++e) n[e] = clamp_count(n[e]);
     }
     for (int gi = 0; gi < p.ntg; ++gi) {
       const int4 d = sD[gi];
@@ -252,6 +280,10 @@ __global__ void __launch_bounds__(NT, MINB) k_schain(const ChainParams p,
       const int4 lo = *reinterpret_cast<const int4 *>(sT + a);
       const int4 hi = *reinterpret_cast<const int4 *>(sT + a + 4);
       sapply<RB>(d.x, v, n, lo, hi, d.w ? nullptr : sN + a);
+      if ((gi & 3) == 3) {
+#pragma unroll
+        for (int e = 0; e < (1 << RB); ++e) n[e] = clamp_count(n[e]);
+      }
     }
     const I bo = rc_base_l<I>(p, tau, p.ssh_out);
     int32_t *dst = C + bo;
@@ -314,9 +346,13 @@ int lead_low_legs(const ChainParams &p, ChainParams *q, int *out) {
 template <int RB, int LWI, int LWO, typename I>
 cudaError_t run(const ChainParams &p, const char *arena, const void *Ax, const uint64_t *An,
                 void *Cx, uint64_t *Cn, const Batch &bt, cudaStream_t st) {
-  constexpr int NT = 128, MINB = RB == 5 ? 3 : 5;
+  constexpr int NT = 128, MINB = 5;
+  // one wave of resident blocks that walk equal numbers of outer indices: every block
+  // builds the gate tables first (a few dependent loads)
   const int64_t need = (p.outer + NT - 1) / NT;
-  const int64_t blocks = wave_blocks(need, bt.B, (int64_t)MINB * num_sms());
+  const int64_t slots = (int64_t)MINB * num_sms();
+  const int64_t trips = (need * bt.B + slots - 1) / slots;
+  const int64_t blocks = (need + trips - 1) / trips;
   k_schain<RB, LWI, LWO, I, NT, MINB><<<dim3((unsigned)blocks, bt.B), NT, 0, st>>>(
       p, reinterpret_cast<const int32_t *>(arena), reinterpret_cast<const uint64_t *>(arena),
       static_cast<const int32_t *>(Ax), An, static_cast<int32_t *>(Cx), Cn, bt.ib);
@@ -351,7 +387,6 @@ cudaError_t launch_schain(const ChainParams &p, const char *arena, const void *A
                           cudaStream_t st) {
   if (p.outer == 0) return cudaSuccess;
   if (p.ntg < 1 || p.P != 1) return cudaErrorInvalidValue;
-  if (p.t == 5) return run_rb<5>(p, arena, Ax, An, Cx, Cn, bt, st);
   if (p.t == 4) return run_rb<4>(p, arena, Ax, An, Cx, Cn, bt, st);
   return cudaErrorInvalidValue;
 }

@@ -47,10 +47,10 @@ __device__ __forceinline__ uint32_t addmod31(uint32_t a, uint32_t b, uint64_t c)
   const uint32_t s = a + b;                            // < 2p < 2^32
   return s >= p ? s - p : s;
 }
-// Exact counts below 2^64 - 1 in one 8-byte plane, saturating: min(n, 2^64 - 1)
-// is compatible with sums and products of counts (which are never negative), so
-// a result below the cap is exact whatever its intermediates did, and one at the
-// cap says that the count needs the residue planes.
+// Exact counts in one 8-byte plane, saturating: min(n, cap) is compatible with sums
+// and products of counts (which are at least 1), so a result below the cap is exact
+// whatever its intermediates did, and one at the cap or above says that the count
+// needs the residue planes.
 __device__ __forceinline__ uint64_t addsat64(uint64_t a, uint64_t b) {
   const uint64_t s = a + b;
   return s < a ? ~0ull : s;

@@ -1168,8 +1168,8 @@ struct Builder {
     kRB = fold ? 6 : 5;
     if (const char *rb = std::getenv("TN_REG_BITS")) kRB = std::max(4, std::min(fold ? 6 : 5, std::atoi(rb)));
     if (P > 0) kRB = 3;
-    // exact 64-bit counts: 12 bytes per state, 2^5 states per thread
-    if (pr.sat && folded()) kRB = std::getenv("TN_SAT_RB") ? std::atoi(std::getenv("TN_SAT_RB")) : 5;
+    // exact 64-bit counts: 12 bytes per state, 2^4 states per thread
+    if (pr.sat && folded()) kRB = 4;
     // integral counts without folding have no register-chain kernel
     if (pr.sat && !folded() && pr.dt == DT_I32) regmode = false;
     if (q == 3) { tmax = 7; wlow = 4; }

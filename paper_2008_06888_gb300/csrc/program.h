@@ -84,7 +84,7 @@ struct Program {
 // budget (PM_CONFIG; <= 0 keeps every intermediate).
 // rbytes: bytes of one residue of the counting planes (8: 61-bit primes; 4:
 // 31-bit primes, the one-prime-per-pass counts).  sat (PM_COUNT, P = 1, rbytes
-// = 8): the plane holds exact counts that saturate at 2^64 - 1.
+// = 8): the plane holds exact, saturating counts.
 bool build_program(const Net &net, const Plan &plan, ProgMode mode, Dtype dt, int P,
                    int64_t seg_bytes, Program *pr, std::string *err, int rbytes = 8,
                    bool sat = false);

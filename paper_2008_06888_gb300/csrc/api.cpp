@@ -102,6 +102,7 @@ const char *op_name(OpKind k) {
     case OP_GEMM: return "maxplus_gemm";
     case OP_TRACE: return "traceback";
     case OP_CHAIN: return "gate_chain";
+    case OP_SMALL: return "small_steps";
   }
   return "op";
 }
@@ -134,12 +135,14 @@ void free_program(Program *p) {
   if (!p) return;
   if (p->d_leaves) cudaFree(p->d_leaves);
   if (p->d_trace) cudaFree(p->d_trace);
+  if (p->d_small) cudaFree(p->d_small);
   if (p->d_chain_traces) cudaFree(p->d_chain_traces);
   for (auto &g : p->graphs)
     if (g.exec) cudaGraphExecDestroy(g.exec);
   p->graphs.clear();
   p->d_leaves = nullptr;
   p->d_trace = nullptr;
+  p->d_small = nullptr;
   p->d_chain_traces = nullptr;
 }
 
@@ -217,6 +220,11 @@ tn_status get_program(tn_ctx *ctx, ProgMode mode, int P, Program **out, int rb =
       CK(cudaMemcpy(p.d_leaves, p.leaves.data(), p.leaves.size() * sizeof(LeafDesc),
                     cudaMemcpyHostToDevice));
     }
+    if (!p.small_desc.empty()) {
+      CK(cudaMalloc(&p.d_small, p.small_desc.size() * sizeof(int32_t)));
+      CK(cudaMemcpy(p.d_small, p.small_desc.data(), p.small_desc.size() * sizeof(int32_t),
+                    cudaMemcpyHostToDevice));
+    }
     if (!p.trace.empty()) {
       CK(cudaMalloc(&p.d_trace, p.trace.size() * sizeof(TraceStep)));
       CK(cudaMemcpy(p.d_trace, p.trace.data(), p.trace.size() * sizeof(TraceStep),
@@ -282,6 +290,7 @@ int op_kind_slot(OpKind k) {
     case OP_LEAVES: return 0;
     case OP_PERM: return 1;
     case OP_GATE: return 2;
+    case OP_SMALL: return 2;
     case OP_GEMM: return 3;
     case OP_TRACE: return 4;
     case OP_CHAIN: return 6;
@@ -361,6 +370,11 @@ tn_status run_ops(tn_ctx *ctx, Program &p, int op_begin, int op_end, cudaStream_
           e = launch_chain(p.dt, p.chains[op.idx], ar, X(op.in0), Nn(op.in0), X(op.out),
                            Nn(op.out), ps, bt, st);
         break;
+      case OP_SMALL: {
+        const SmallRun &r = p.smalls[op.idx];
+        e = launch_small(p.dt, p.sat, p.d_small + r.desc_off, r.desc_len, ar, bt, st);
+        break;
+      }
     }
     if (e != cudaSuccess)
       return fail(ctx, TN_ECUDA, std::string("kernel launch: ") + cudaGetErrorString(e));
@@ -824,7 +838,8 @@ tn_status tn_order(tn_ctx *ctx, int32_t method, const int32_t *seq, int32_t seq_
     auto score = [&](const Plan &pl) -> double {
       Program pg;
       std::string e2;
-      if (!build_program(ctx->net, pl, PM_ENERGY, dt, 0, 0, &pg, &e2)) return INFINITY;
+      if (!build_program(ctx->net, pl, PM_ENERGY, dt, 0, 0, &pg, &e2, 8, false, false))
+        return INFINITY;
       double tsec = 0;
       for (const Op &op : pg.ops) {
         tsec += 2.0e-6;  // launch / latency floor per kernel in a graph
@@ -1599,7 +1614,10 @@ tn_status tn_energy_noalloc(tn_ctx *ctx, const float *J_dev, const float *h_dev,
   if (!ctx->prog_noalloc || ctx->noalloc_fp != fp) {
     std::unique_ptr<Program> pg(new Program());
     std::string err;
-    if (!build_program(ctx->net, ctx->plan, PM_ENERGY, ctx->dt, 0, 0, pg.get(), &err))
+    // (its steps travel as kernel parameters: no runs, whose descriptors would need
+    // device memory)
+    if (!build_program(ctx->net, ctx->plan, PM_ENERGY, ctx->dt, 0, 0, pg.get(), &err, 8, false,
+                       false))
       return fail(ctx, TN_EINVAL, err);
     ctx->prog_noalloc = std::move(pg);
     ctx->noalloc_fp = fp;
@@ -1643,6 +1661,7 @@ tn_status tn_energy_noalloc(tn_ctx *ctx, const float *J_dev, const float *h_dev,
         e = launch_mpgemm(p.dt, p.gemms[op.idx], X(op.in0), X(op.in1), X(op.out), one, st);
         break;
       case OP_TRACE:
+      case OP_SMALL:
         break;
       case OP_CHAIN:
         e = launch_chain(p.dt, p.chains[op.idx], base, X(op.in0), nullptr, X(op.out), nullptr, ps,

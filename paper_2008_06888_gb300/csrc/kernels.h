@@ -3,6 +3,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <vector>
+
 #include "tn_internal.h"
 
 namespace tn {
@@ -68,6 +70,17 @@ cudaError_t launch_trace(Dtype dt, int q, const TraceStep *d_steps, int nsteps,
                          const ChainTrace *d_chains, size_t smem, const char *arena, int8_t *state,
                          int nspins, int *err, const Batch &bt, cudaStream_t st);
 size_t trace_smem_bytes(const ChainParams &p, size_t elem);
+
+// A run of small steps in one launch, one block per instance.  Descriptors (32-bit
+// words): {steps, levels}, level starts [levels + 1], per step its first output within
+// its level, per step the word of its body, then the bodies: 64-bit offsets of the
+// values of A, B (-1: none) and C in elements and of their counts in 8-byte words,
+// digits, K, N, unit B counts, outputs, then (size, stride in A, stride in B) of each
+// outer digit (slowest first), (offset in A, in B) of each k, the offset in B of each n.
+// sat: one plane of saturating 64-bit counts.
+constexpr int kSmallMaxWords = 40 * 1024;     // descriptor words of a run at most
+cudaError_t launch_small(Dtype dt, bool sat, const int32_t *d_desc, int words, char *arena,
+                         const Batch &bt, cudaStream_t st);
 
 // Fused gate chain over tiles of the big tensor (values; planes when P > 0).
 cudaError_t launch_chain(Dtype dt, const ChainParams &p, const char *arena, const void *Ax,

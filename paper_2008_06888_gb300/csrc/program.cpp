@@ -198,6 +198,8 @@ struct Builder {
   // nothing from unit inputs: outer products and Hadamard-type steps)
   std::vector<char> unit;
 
+  bool small_runs = true;
+
   Builder(const Net &n, const Plan &p, Program &r)
       : net(n), plan(p), pr(r), q(r.q), P(r.P), rb(r.rbytes), order(p.legset.size()),
         loc(p.legset.size()),
@@ -226,8 +228,10 @@ struct Builder {
     l.plane = elems;
     return l;
   }
+  std::vector<std::pair<int, int>> uses;   // every (op, buffer)
   void use(const Loc &l, int op) {
     if (l.buf < 0) return;
+    uses.push_back({op, l.buf});
     BufInfo &b = pr.bufs[l.buf];
     b.first = std::min(b.first, op);
     b.last = std::max(b.last, op);
@@ -1156,6 +1160,112 @@ struct Builder {
     return true;
   }
 
+  // ---- runs of small steps (SmallRun)
+  //
+  // A step counts as small up to kSmallWork products: at that size one block takes
+  // about as long as a kernel launch (~2 us).
+  static constexpr int64_t kSmallWork = 4096;
+  bool small_step(const Op &op) const {
+    if (op.kind == OP_GATE) {
+      const GateParams &g = pr.gates[op.idx];
+      return g.outer * g.Ks * g.Ns <= kSmallWork;
+    }
+    if (op.kind == OP_PERM) return pr.perms[op.idx].total <= kSmallWork && pr.perms[op.idx].r <= 14;
+    if (op.kind == OP_GEMM) {
+      const GemmParams &g = pr.gemms[op.idx];
+      return g.K <= 64 && g.batch * g.M * g.N * g.K <= kSmallWork;
+    }
+    return false;
+  }
+  int small_words(const Op &op) const {   // an upper bound of its descriptor
+    const int seg = op.kind == OP_GATE ? pr.gates[op.idx].nseg : op.kind == OP_PERM ? 14 : 3;
+    const int ks = op.kind == OP_GATE ? pr.gates[op.idx].Ks : op.kind == OP_GEMM ? 64 : 1;
+    return 24 + 3 * seg + 2 * ks + TN_GATE_MAX_N;
+  }
+
+  // Every small step of the forward pass moves up to right behind the last launch it
+  // depends on, and the small steps behind one launch become one run, sorted by
+  // dependency level.  Steps keep their operands and arithmetic.
+  void schedule_small() {
+    const int F = pr.fwd_end;
+    std::vector<int> prod(pr.bufs.size(), -1);     // forward op writing each buffer
+    for (int i = 0; i < F; ++i)
+      if (pr.ops[i].out.buf >= 0) prod[pr.ops[i].out.buf] = i;
+    std::vector<std::vector<int>> in(F);
+    for (auto &u : uses)
+      if (u.first < F && pr.ops[u.first].out.buf != u.second && prod[u.second] >= 0)
+        in[u.first].push_back(prod[u.second]);
+    std::vector<int> stage(F, 0), level(F, 0), bigs;
+    std::vector<char> small(F, 0);
+    for (int i = 0; i < F; ++i) {
+      small[i] = small_step(pr.ops[i]);
+      if (!small[i]) {
+        stage[i] = (int)bigs.size();
+        bigs.push_back(i);
+        continue;
+      }
+      for (int d : in[i]) stage[i] = std::max(stage[i], stage[d]);
+      for (int d : in[i])
+        if (small[d] && stage[d] == stage[i]) level[i] = std::max(level[i], level[d] + 1);
+    }
+    std::vector<std::vector<int>> after(bigs.size());
+    for (int i = 0; i < F; ++i)
+      if (small[i]) after[stage[i]].push_back(i);
+    std::vector<Op> ops;
+    std::vector<int> at(pr.ops.size() + 1);
+    for (size_t b = 0; b < bigs.size(); ++b) {
+      at[bigs[b]] = (int)ops.size();
+      ops.push_back(pr.ops[bigs[b]]);
+      std::vector<int> &run = after[b];
+      std::stable_sort(run.begin(), run.end(), [&](int x, int y) { return level[x] < level[y]; });
+      for (size_t k = 0; k < run.size();) {
+        SmallRun sr;
+        int words = 8;
+        size_t e = k;
+        for (; e < run.size(); ++e) {
+          const int w = small_words(pr.ops[run[e]]) + 3;
+          if (words + w > kSmallMaxWords) break;
+          words += w;
+        }
+        if (e - k == 1) {   // a step by itself keeps its own kernel
+          at[run[k]] = (int)ops.size();
+          ops.push_back(pr.ops[run[k]]);
+          k = e;
+          continue;
+        }
+        Op op;
+        op.kind = OP_SMALL;
+        op.idx = (int)pr.smalls.size();
+        for (size_t j = k; j < e; ++j) {
+          const Op &o = pr.ops[run[j]];
+          if (j == k || level[run[j]] != level[run[j - 1]]) sr.level.push_back((int)(j - k));
+          sr.ops.push_back(o);
+          at[run[j]] = (int)ops.size();
+          op.bytes += o.bytes;
+          op.macs += o.macs;
+        }
+        sr.level.push_back((int)sr.ops.size());
+        pr.smalls.push_back(sr);
+        ops.push_back(op);
+        k = e;
+      }
+    }
+    pr.fwd_end = (int)ops.size();
+    for (size_t i = F; i < pr.ops.size(); ++i) {
+      at[i] = (int)ops.size();
+      ops.push_back(pr.ops[i]);
+    }
+    at[pr.ops.size()] = (int)ops.size();
+    pr.ops.swap(ops);
+    // the steps of a run share one place in time, so no two of their buffers overlap
+    for (BufInfo &b : pr.bufs) { b.first = 1 << 30; b.last = -1; }
+    for (auto &u : uses) {
+      BufInfo &b = pr.bufs[u.second];
+      b.first = std::min(b.first, at[u.first]);
+      b.last = std::max(b.last, at[u.first]);
+    }
+  }
+
   bool build(ProgMode mode, int64_t seg_bytes) {
     fuse = std::getenv("TN_NO_FUSION") == nullptr;
     // register chains: q = 2 values, or q = 2 counts with 3 primes + witness
@@ -1203,6 +1313,8 @@ struct Builder {
       flush_trace();
     }
     use(pr.root, (int)pr.ops.size());
+    if (small_runs && (P == 0 || pr.sat) && std::getenv("TN_NO_SMALL_RUNS") == nullptr)
+      schedule_small();
     return true;
   }
 };
@@ -1240,8 +1352,109 @@ void plan_memory(Program &pr) {
 
 int64_t abs_off(const Program &pr, const Loc &l) { return pr.bufs[l.buf].off + l.xoff; }
 
+struct SmallBody {
+  int64_t offA = 0, offB = -1, offC = 0;   // element offsets of the values (B: -1 none)
+  int64_t nA = 0, nB = 0, nC = 0;          // and of the counts, in 8-byte words
+  int nout = 0, unitB = 1;
+  int Ks = 1, Ns = 1;
+  std::vector<int64_t> seg_size, seg_sA, seg_sB;   // outer digits, slowest first
+  std::vector<int64_t> kA, kB, nBo;        // offsets of k in A and B, of n in B
+};
+
+// descriptors of a run, laid out as k_small reads them (kernels.h)
+static std::vector<int32_t> encode_small(const std::vector<SmallBody> &ops,
+                                         const std::vector<int> &level) {
+  const int n = (int)ops.size(), nlev = (int)level.size() - 1;
+  std::vector<int32_t> w{n, nlev};
+  w.insert(w.end(), level.begin(), level.end());
+  const size_t first = w.size(), body = first + n;
+  w.resize(body + n);
+  auto put64 = [&](int64_t v) {
+    w.push_back((int32_t)(uint32_t)(uint64_t)v);
+    w.push_back((int32_t)(uint32_t)((uint64_t)v >> 32));
+  };
+  for (int l = 0; l < nlev; ++l) {
+    int at = 0;
+    for (int i = level[l]; i < level[l + 1]; ++i) {
+      const SmallBody &o = ops[i];
+      w[first + i] = at;
+      w[body + i] = (int32_t)w.size();
+      at += o.nout;
+      for (int64_t v : {o.offA, o.offB, o.offC, o.nA, o.nB, o.nC}) put64(v);
+      w.push_back((int32_t)o.seg_size.size());
+      w.push_back(o.Ks);
+      w.push_back(o.Ns);
+      w.push_back(o.unitB);
+      w.push_back(o.nout);
+      for (size_t s = 0; s < o.seg_size.size(); ++s) {
+        w.push_back((int32_t)o.seg_size[s]);
+        w.push_back((int32_t)o.seg_sA[s]);
+        w.push_back((int32_t)o.seg_sB[s]);
+      }
+      for (int k = 0; k < o.Ks; ++k) {
+        w.push_back((int32_t)o.kA[k]);
+        w.push_back((int32_t)o.kB[k]);
+      }
+      if (o.Ns > 1)
+        for (int k = 0; k < o.Ns; ++k) w.push_back((int32_t)o.nBo[k]);
+    }
+  }
+  return w;
+}
+
+// a small step with its planned offsets
+static SmallBody small_body(const Program &pr, const Op &op) {
+  SmallBody b;
+  auto cnt = [&](const Loc &l) { return (pr.bufs[l.buf].off + l.noff) / 8; };
+  b.offA = abs_off(pr, op.in0) / 4;
+  b.offC = abs_off(pr, op.out) / 4;
+  b.offB = op.in1.buf >= 0 ? abs_off(pr, op.in1) / 4 : -1;
+  if (pr.sat) {
+    b.nA = cnt(op.in0);
+    b.nC = cnt(op.out);
+    b.nB = op.in1.buf >= 0 ? cnt(op.in1) : 0;
+  }
+  auto digit = [&](int64_t size, int64_t sA, int64_t sB) {
+    b.seg_size.push_back(size);
+    b.seg_sA.push_back(sA);
+    b.seg_sB.push_back(sB);
+  };
+  if (op.kind == OP_GATE) {
+    const GateParams &g = pr.gates[op.idx];
+    for (int s = 0; s < g.nseg; ++s) digit(g.seg_size[s], g.seg_sA[s], g.seg_sB[s]);
+    b.Ks = g.Ks;
+    b.Ns = g.Ns;
+    b.unitB = g.unitB;
+    b.nout = (int)(g.outer * g.Ns);
+    b.kA.assign(g.kA, g.kA + g.Ks);
+    b.kB.assign(g.kB, g.kB + g.Ks);
+    b.nBo.assign(g.nB, g.nB + g.Ns);
+    if (!g.hasB) b.offB = -1;
+  } else if (op.kind == OP_PERM) {
+    const PermParams &p = pr.perms[op.idx];
+    for (int s = 0; s < p.r; ++s) digit(p.dims[s], p.sin[s], 0);
+    b.nout = (int)p.total;
+    b.kA = b.kB = b.nBo = {0};
+  } else {
+    const GemmParams &g = pr.gemms[op.idx];
+    digit(g.batch, g.sAb, g.sBb);
+    digit(g.M, g.sAm, 0);
+    digit(g.N, 0, g.sBn);
+    b.nout = (int)(g.batch * g.M * g.N);
+    b.Ks = (int)g.K;
+    b.unitB = 0;
+    for (int64_t k = 0; k < g.K; ++k) {
+      b.kA.push_back(k * g.sAk);
+      b.kB.push_back(k * g.sBk);
+    }
+    b.nBo = {0};
+  }
+  return b;
+}
+
 bool build_program(const Net &net, const Plan &plan, ProgMode mode, Dtype dt, int P,
-                   int64_t seg_bytes, Program *pr, std::string *err, int rbytes, bool sat) {
+                   int64_t seg_bytes, Program *pr, std::string *err, int rbytes, bool sat,
+                   bool small_runs) {
   *pr = Program();
   pr->mode = mode;
   pr->dt = dt;
@@ -1258,6 +1471,7 @@ bool build_program(const Net &net, const Plan &plan, ProgMode mode, Dtype dt, in
   pr->rbytes = rbytes;
   pr->sat = sat;
   Builder bd(net, plan, *pr);
+  bd.small_runs = small_runs;
   if (!bd.build(mode, seg_bytes)) {
     *err = bd.err.empty() ? "program: lowering failed" : bd.err;
     return false;
@@ -1267,8 +1481,17 @@ bool build_program(const Net &net, const Plan &plan, ProgMode mode, Dtype dt, in
     // "1": every program built; "c": only traceback / counting programs
     if (*dump == '1' || (*dump == 'c' && mode != PM_ENERGY)) {
       std::fprintf(stderr, "program mode %d ops %zu\n", (int)mode, pr->ops.size());
-      for (size_t i = 0; i < pr->ops.size(); ++i) {
-        const Op &o = pr->ops[i];
+      std::vector<Op> all;   // the steps of small runs listed one by one
+      for (const Op &o : pr->ops) {
+        if (o.kind == OP_SMALL) {
+          const SmallRun &r = pr->smalls[o.idx];
+          all.insert(all.end(), r.ops.begin(), r.ops.end());
+        } else {
+          all.push_back(o);
+        }
+      }
+      for (size_t i = 0; i < all.size(); ++i) {
+        const Op &o = all[i];
         std::fprintf(stderr, "op %zu kind %d bytes %.0f in0 %lld in1 %lld out %lld", i, (int)o.kind,
                      o.bytes,
                      (long long)(o.in0.buf >= 0 ? o.in0.plane : -1),
@@ -1315,6 +1538,15 @@ bool build_program(const Net &net, const Plan &plan, ProgMode mode, Dtype dt, in
         std::fprintf(stderr, "\n");
       }
     }
+  }
+  // descriptors of the small runs
+  for (SmallRun &r : pr->smalls) {
+    std::vector<SmallBody> bodies;
+    for (const Op &op : r.ops) bodies.push_back(small_body(*pr, op));
+    const std::vector<int32_t> w = encode_small(bodies, r.level);
+    r.desc_off = (int64_t)pr->small_desc.size();
+    r.desc_len = (int)w.size();
+    pr->small_desc.insert(pr->small_desc.end(), w.begin(), w.end());
   }
   // absolute offsets of leaves and traceback operands
   const int64_t lbase = pr->bufs[pr->leaves_loc.buf].off;

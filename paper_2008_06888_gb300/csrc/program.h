@@ -24,7 +24,7 @@ struct BufInfo {
   int64_t off = -1;
 };
 
-enum OpKind { OP_LEAVES, OP_PERM, OP_GATE, OP_GEMM, OP_TRACE, OP_CHAIN };
+enum OpKind { OP_LEAVES, OP_PERM, OP_GATE, OP_GEMM, OP_TRACE, OP_CHAIN, OP_SMALL };
 
 struct Op {
   OpKind kind;
@@ -32,6 +32,17 @@ struct Op {
   int idx = -1;              // into gates / gemms / perms
   int trace_begin = 0, trace_n = 0;
   double bytes = 0, macs = 0;  // algorithmic traffic and multiply-adds of the launch
+};
+
+// A run of small steps (gates, transposes, GEMMs of few elements) that one block per
+// instance executes in one launch: ops sorted by dependency level, level l being
+// ops [level[l], level[l + 1]).  The encoded descriptors (kernels.h) start at int
+// desc_off of the program's descriptor array.
+struct SmallRun {
+  std::vector<Op> ops;
+  std::vector<int> level;
+  int64_t desc_off = 0;
+  int desc_len = 0;
 };
 
 enum ProgMode { PM_ENERGY = 0, PM_CONFIG = 1, PM_COUNT = 2 };
@@ -48,6 +59,8 @@ struct Program {
   std::vector<GateParams> gates;
   std::vector<GemmParams> gemms;
   std::vector<PermParams> perms;
+  std::vector<SmallRun> smalls;
+  std::vector<int32_t> small_desc;                  // descriptors of every run
   std::vector<ChainParams> chains;                  // fused gate chains
   std::vector<const void *> chain_jit;              // their compiled kernels (nullptr: interpreted)
   std::vector<std::vector<Loc>> chain_blocs;        // their gate operands
@@ -76,6 +89,7 @@ struct Program {
   std::vector<Graph> graphs;
   // device copies (owned by the context)
   LeafDesc *d_leaves = nullptr;
+  int32_t *d_small = nullptr;
   TraceStep *d_trace = nullptr;
   ChainTrace *d_chain_traces = nullptr;
 };
@@ -84,10 +98,11 @@ struct Program {
 // budget (PM_CONFIG; <= 0 keeps every intermediate).
 // rbytes: bytes of one residue of the counting planes (8: 61-bit primes; 4:
 // 31-bit primes, the one-prime-per-pass counts).  sat (PM_COUNT, P = 1, rbytes
-// = 8): the plane holds exact, saturating counts.
+// = 8): the plane holds exact, saturating counts.  small_runs: group the small
+// steps of the forward pass into runs (value and exact-count programs).
 bool build_program(const Net &net, const Plan &plan, ProgMode mode, Dtype dt, int P,
                    int64_t seg_bytes, Program *pr, std::string *err, int rbytes = 8,
-                   bool sat = false);
+                   bool sat = false, bool small_runs = true);
 
 int64_t abs_off(const Program &pr, const Loc &l);  // arena byte offset of values
 

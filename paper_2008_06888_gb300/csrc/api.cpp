@@ -136,13 +136,17 @@ void free_program(Program *p) {
   if (p->d_leaves) cudaFree(p->d_leaves);
   if (p->d_trace) cudaFree(p->d_trace);
   if (p->d_small) cudaFree(p->d_small);
+  if (p->d_walk) cudaFree(p->d_walk);
+  if (p->d_walk_idx) cudaFree(p->d_walk_idx);
+  if (p->d_walk_list) cudaFree(p->d_walk_list);
   if (p->d_chain_traces) cudaFree(p->d_chain_traces);
   for (auto &g : p->graphs)
     if (g.exec) cudaGraphExecDestroy(g.exec);
   p->graphs.clear();
   p->d_leaves = nullptr;
   p->d_trace = nullptr;
-  p->d_small = nullptr;
+  p->d_small = p->d_walk = p->d_walk_list = nullptr;
+  p->d_walk_idx = nullptr;
   p->d_chain_traces = nullptr;
 }
 
@@ -184,6 +188,15 @@ tn_status ensure_device(tn_ctx *ctx) {
   return TN_OK;
 }
 
+// a device copy of v (none when it is empty)
+template <typename V>
+cudaError_t to_device(const std::vector<V> &v, V **d) {
+  if (v.empty()) return cudaSuccess;
+  cudaError_t e = cudaMalloc(d, v.size() * sizeof(V));
+  if (e != cudaSuccess) return e;
+  return cudaMemcpy(*d, v.data(), v.size() * sizeof(V), cudaMemcpyHostToDevice);
+}
+
 tn_status get_program(tn_ctx *ctx, ProgMode mode, int P, Program **out, int rb = 8,
                       bool sat = false) {
   if (!ctx->ordered) return fail(ctx, TN_ESTATE, "tn_order has not been called");
@@ -215,26 +228,13 @@ tn_status get_program(tn_ctx *ctx, ProgMode mode, int P, Program **out, int rb =
       return fail(ctx, TN_EINVAL, err);
     }
     Program &p = *slot;
-    if (!p.leaves.empty()) {
-      CK(cudaMalloc(&p.d_leaves, p.leaves.size() * sizeof(LeafDesc)));
-      CK(cudaMemcpy(p.d_leaves, p.leaves.data(), p.leaves.size() * sizeof(LeafDesc),
-                    cudaMemcpyHostToDevice));
-    }
-    if (!p.small_desc.empty()) {
-      CK(cudaMalloc(&p.d_small, p.small_desc.size() * sizeof(int32_t)));
-      CK(cudaMemcpy(p.d_small, p.small_desc.data(), p.small_desc.size() * sizeof(int32_t),
-                    cudaMemcpyHostToDevice));
-    }
-    if (!p.trace.empty()) {
-      CK(cudaMalloc(&p.d_trace, p.trace.size() * sizeof(TraceStep)));
-      CK(cudaMemcpy(p.d_trace, p.trace.data(), p.trace.size() * sizeof(TraceStep),
-                    cudaMemcpyHostToDevice));
-    }
-    if (!p.chain_traces.empty()) {
-      CK(cudaMalloc(&p.d_chain_traces, p.chain_traces.size() * sizeof(ChainTrace)));
-      CK(cudaMemcpy(p.d_chain_traces, p.chain_traces.data(),
-                    p.chain_traces.size() * sizeof(ChainTrace), cudaMemcpyHostToDevice));
-    }
+    CK(to_device(p.leaves, &p.d_leaves));
+    CK(to_device(p.small_desc, &p.d_small));
+    if (p.walks.empty()) CK(to_device(p.trace, &p.d_trace));
+    CK(to_device(p.chain_traces, &p.d_chain_traces));
+    CK(to_device(p.walk_words, &p.d_walk));
+    CK(to_device(p.walk_idx, &p.d_walk_idx));
+    CK(to_device(p.walk_list, &p.d_walk_list));
     if (mode == PM_COUNT && !sat) {
       ctx->prog_P = P;
       ctx->prog_rb = rb;
@@ -359,6 +359,23 @@ tn_status run_ops(tn_ctx *ctx, Program &p, int op_begin, int op_end, cudaStream_
                                 Nn(op.in0), Nn(op.in1), Nn(op.out), ps, bt, st);
         break;
       case OP_TRACE:
+        if (op.idx >= 0) {
+          const Walk &w = p.walks[op.idx];
+          WalkArgs a;
+          a.recs = p.d_walk;
+          a.idx = p.d_walk_idx + w.idx_off;
+          a.n = w.n;
+          a.list = p.d_walk_list + w.list_off;
+          a.nlist = w.nlist;
+          a.chains = p.d_chain_traces;
+          a.best = w.best.buf >= 0 ? abs_off(p, w.best) : -1;
+          a.nbig = (int)w.big.size();
+          a.big = w.big.data();
+          a.big_rec = w.big_rec.data();
+          a.big_k = w.big_k.data();
+          e = launch_walk(p.dt, a, ar, ra.state, ctx->net.n, ctx->d_err, bt, st);
+          break;
+        }
         e = launch_trace(p.dt, p.q, p.d_trace + op.trace_begin, op.trace_n, p.d_chain_traces,
                          p.trace_smem, ar, ra.state, ctx->net.n, ctx->d_err, bt, st);
         break;

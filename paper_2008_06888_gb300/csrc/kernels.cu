@@ -2636,105 +2636,10 @@ cudaError_t launch_rchain_count(Dtype dt, const ChainParams &p, const char *aren
   return cudaGetLastError();
 }
 
-// Traceback of a register chain by one warp: lane e holds element e of the
+// Traceback of an unfolded register chain by one warp: lane e holds element e of the
 // 2^t elements of the fixed outer index; the gates are replayed (every
 // intermediate kept in shared memory) with the forward's operation order,
 // then lane 0 undoes each replace gate with the first-index argmax.
-// Traceback of a folded register chain: the 32 elements selected by the
-// outer spins are recomputed through the table gates in a warp (the same
-// sums as the forward kernel), then walked backwards through the replace
-// gates; ties keep the contracted digit 0.
-template <typename T>
-__device__ void trace_tchain(const ChainTrace &ct, const T *X, int8_t *state, int *err, T *buf,
-                             T *sT) {
-  const ChainParams &p = ct.p;
-  const int E = p.tile;
-  build_tables<T>(p, X, sT);
-  __syncthreads();
-  const int lane = threadIdx.x & 31;
-  if (threadIdx.x < 32) {
-    int64_t part = 0, tpart = 0;   // input offset and outer index tau of the outer spins
-    for (int i = lane; i < ct.nout; i += 32) {
-      int d = state[ct.out_spin[i]];
-      if (d < 0 || d > 1) { *err = 1; d = 0; }
-      part += (int64_t)d * ct.out_stride[i];
-      tpart += (int64_t)d << ct.out_rank[i];
-    }
-    for (int o = 16; o > 0; o >>= 1) {
-      part += __shfl_xor_sync(0xffffffffu, part, o);
-      tpart += __shfl_xor_sync(0xffffffffu, tpart, o);
-    }
-    const int64_t base = part, tau = tpart;
-    auto slice = [&](const TGate &t) {
-      int f = 0;
-      for (int i = 0; i < t.nf; ++i) f |= (int)((tau >> t.fsh[i]) & 1) << i;
-      return sT + t.toff + f * 8;
-    };
-    for (int e = lane; e < E; e += 32) buf[e] = X[ct.offIn + base + p.hi_in[e]];
-    __syncwarp();
-    for (int gi = 0; gi < p.ntg; ++gi) {
-      const TGate &t = p.tg[gi];
-      const T *src = buf + (int64_t)gi * E;
-      T *dst = buf + (int64_t)(gi + 1) * E;
-      const T *tab = slice(t);
-      for (int e = lane; e < E; e += 32) {
-        if (t.kind == 2) {   // final contraction: states with bit J clear
-          if (!(e & (1 << t.J))) {
-            const int k = t.K >= 0 ? (e >> t.K) & 1 : 0;
-            dst[e] = max(src[e] + tab[k * 4], src[e | (1 << t.J)] + tab[k * 4 + 1]);
-          }
-        } else if (t.kind != 0) {
-          const int x0 = t.J >= 0 ? (e >> t.J) & 1 : 0, x1 = t.K >= 0 ? (e >> t.K) & 1 : 0;
-          dst[e] = src[e] + tab[x0 | (x1 << 1)];
-        } else if (!(e & (1 << t.J))) {
-          const int e1 = e | (1 << t.J);
-          const int k = t.K >= 0 ? (e >> t.K) & 1 : 0;
-          const T a = src[e], b = src[e1];
-          dst[e] = max(a + tab[k * 4 + 0], b + tab[k * 4 + 1]);
-          dst[e1] = max(a + tab[k * 4 + 2], b + tab[k * 4 + 3]);
-        }
-      }
-      __syncwarp();
-    }
-    if (lane == 0) {
-      // a final contraction's leg is not fixed yet: its digit is chosen first
-      const int cj = p.ntg > 0 && p.tg[p.ntg - 1].kind == 2 ? p.tg[p.ntg - 1].J : -1;
-      int x = 0;
-      for (int j = 0; j < p.t; ++j) {
-        if (j == cj) continue;
-        int d = state[ct.local_spin[j]];
-        if (d < 0 || d > 1) { *err = 1; d = 0; }
-        x |= d << j;
-      }
-      for (int gi = p.ntg - 1; gi >= 0; --gi) {
-        const TGate &t = p.tg[gi];
-        if (t.kind == 2) {
-          const T *src = buf + (int64_t)gi * E;
-          const T *tab = slice(t);
-          const int k = t.K >= 0 ? (x >> t.K) & 1 : 0;
-          const T c0 = src[x] + tab[k * 4], c1 = src[x | (1 << t.J)] + tab[k * 4 + 1];
-          const int u = c1 > c0 ? 1 : 0;
-          state[t.kspin] = (int8_t)u;
-          x |= u << t.J;
-          continue;
-        }
-        if (t.kind != 0) continue;
-        const T *src = buf + (int64_t)gi * E;
-        const T *tab = slice(t);
-        const int v = (x >> t.J) & 1;
-        const int x0 = x & ~(1 << t.J);
-        const int k = t.K >= 0 ? (x0 >> t.K) & 1 : 0;
-        const T c0 = src[x0] + tab[k * 4 + v * 2 + 0];
-        const T c1 = src[x0 | (1 << t.J)] + tab[k * 4 + v * 2 + 1];
-        const int u = c1 > c0 ? 1 : 0;
-        state[t.kspin] = (int8_t)u;
-        x = x0 | (u << t.J);
-      }
-    }
-  }
-  __syncthreads();
-}
-
 template <typename T>
 __device__ void trace_rchain(const ChainTrace &ct, const T *X, int8_t *state, int *err,
                              char *smem, int64_t *sbase) {
@@ -2742,10 +2647,6 @@ __device__ void trace_rchain(const ChainTrace &ct, const T *X, int8_t *state, in
   const int E = p.tile;   // 32
   T *buf = reinterpret_cast<T *>(smem);
   T *sBg = buf + (int64_t)(p.ngates + 1) * E;   // staged gate operands
-  if (p.ntg > 0) {
-    trace_tchain<T>(ct, X, state, err, buf, sBg);
-    return;
-  }
   load_gate_operands<T, uint64_t>(p, X, nullptr, sBg, nullptr, kGateBMax);
   __syncthreads();
   const int lane = threadIdx.x & 31;
@@ -2932,8 +2833,8 @@ __device__ __forceinline__ void argmax_merge(T &v, int &k, T v2, int k2) {
   }
 }
 
-// One block walks the records in order (the host lists them top-down).  The
-// spin state lives in shared memory (`sst`) for the whole walk.  Plain
+// One block walks the records in order (the host lists them top-down): Potts plans and
+// q = 2 plans without folded chains (trace_walk.cu has the others).  The spin state lives in shared memory (`sst`) for the whole walk.  Plain
 // records: the fixed legs select a slice of A and B, the block finds the first
 // k maximising A + B and assigns the contracted spins.  Chain records:
 // trace_chain above.

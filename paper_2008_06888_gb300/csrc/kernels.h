@@ -71,6 +71,31 @@ cudaError_t launch_trace(Dtype dt, int q, const TraceStep *d_steps, int nsteps,
                          int nspins, int *err, const Batch &bt, cudaStream_t st);
 size_t trace_smem_bytes(const ChainParams &p, size_t elem);
 
+// The traceback of q = 2 plans whose chains are folded (trace_walk.cu).  A record is a
+// list of 32-bit words (encode_walk in program.cpp); tab: element offset of a chain
+// record's gate tables in the instance's arena slice (ntab values).
+constexpr int kWalkTable = TN_CHAIN_MAX_G * TN_TG_TABLE;
+constexpr int kWalkRec = 8 + 7 * TN_MAX_TRACE_LEGS;
+struct WalkIdx {
+  int64_t tab;
+  int32_t rec, len, ntab, pad;
+};
+struct WalkArgs {
+  const int32_t *recs = nullptr;       // device: record words
+  const WalkIdx *idx = nullptr;        // device: this trace's records
+  int n = 0;
+  const int32_t *list = nullptr;       // device: (record, chain) of its chain records
+  int nlist = 0;
+  const ChainTrace *chains = nullptr;  // device
+  int64_t best = -1;                   // arena byte offset of the wide search's key
+  // records searched by a grid, in order: position, record word, contracted states
+  int nbig = 0;
+  const int *big = nullptr, *big_rec = nullptr;
+  const int64_t *big_k = nullptr;
+};
+cudaError_t launch_walk(Dtype dt, const WalkArgs &w, char *arena, int8_t *state, int nspins,
+                        int *err, const Batch &bt, cudaStream_t st);
+
 // A run of small steps in one launch, one block per instance.  Descriptors (32-bit
 // words): {steps, levels}, level starts [levels + 1], per step its first output within
 // its level, per step the word of its body, then the bodies: 64-bit offsets of the

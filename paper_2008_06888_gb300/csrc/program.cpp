@@ -1077,11 +1077,11 @@ struct Builder {
     Op op;
     op.kind = OP_TRACE;
     op.trace_begin = (int)pr.trace.size();
-    op.trace_n = (int)pending.size();
     pr.ops.push_back(op);
     int oi = (int)pr.ops.size() - 1;
     for (int mi : pending) {
       const Macro &m = macros[mi];
+      if (!chooses(m)) continue;
       TraceStep t{};
       t.chain = -1;
       if (m.chain) {
@@ -1145,6 +1145,39 @@ struct Builder {
       if (st.b >= 0) use(loc[st.b], oi);
     }
     pending.clear();
+    pr.ops[oi].trace_n = (int)pr.trace.size() - pr.ops[oi].trace_begin;
+    if (q == 2 && regmode && folded()) add_walk(oi);
+  }
+
+  // a macro that contracts no leg fixes no spin: the traceback has nothing to do there
+  bool chooses(const Macro &m) const { return m.chain || !plan.steps[m.step].K.empty(); }
+
+  // Steps with at least this many contracted states are searched by a grid of their own
+  // (a warp takes about 10 us for 1024, a grid about 5 us).
+  static constexpr int64_t kWalkBig = 1024;
+  void add_walk(int oi) {
+    Op &op = pr.ops[oi];
+    Walk w;
+    w.begin = op.trace_begin;
+    w.n = op.trace_n;
+    int64_t tables = 0;
+    bool big = false;
+    for (int i = 0; i < w.n; ++i) {
+      const TraceStep &t = pr.trace[w.begin + i];
+      w.toff.push_back(tables);
+      if (t.chain >= 0) tables += pr.chain_traces[t.chain].p.ttotal;
+      big = big || (t.chain < 0 && t.Ks >= kWalkBig);
+    }
+    if (tables > 0) {
+      w.tables = new_tensor(tables);
+      use(w.tables, oi);
+    }
+    if (big) {
+      w.best = new_tensor(2);
+      use(w.best, oi);
+    }
+    op.idx = (int)pr.walks.size();
+    pr.walks.push_back(w);
   }
 
   std::vector<char> avail;
@@ -1301,6 +1334,7 @@ struct Builder {
       }
       avail = stored;
       for (int mi = (int)macros.size() - 1; mi >= 0; --mi) {
+        if (!chooses(macros[mi])) continue;
         bool need = false;
         for (int x : macro_inputs(macros[mi])) need = need || !avail[x];
         if (need) {
@@ -1400,6 +1434,62 @@ static std::vector<int32_t> encode_small(const std::vector<SmallBody> &ops,
     }
   }
   return w;
+}
+
+// One traceback record as k_walk reads it.  Plain: {0, legs of A, legs of B, contracted
+// legs, offset of A (2 words), of B (2, -1: none)}, then (spin, log2 stride) of the fixed
+// legs of A and of B, then (spin, log2 stride in A, in B) of the contracted ones.  Chain:
+// {1, outer legs, register legs, gates, offset of the input (2), 0, 0, spin of each
+// register leg [6], its log2 stride in the input [6; 63: none]}, then (spin, log2 stride,
+// bit in the outer index) of the outer legs, then per gate {kind | J + 1 | K + 1, bits of
+// its fixed legs, table offset, contracted spin}.
+static void encode_walk(const Program &pr, const TraceStep &t, std::vector<int32_t> *w) {
+  auto put64 = [&](int64_t v) {
+    w->push_back((int32_t)(uint32_t)(uint64_t)v);
+    w->push_back((int32_t)(uint32_t)((uint64_t)v >> 32));
+  };
+  auto lg = [](int64_t x) { int r = 0; while ((int64_t(1) << r) < x) ++r; return r; };
+  if (t.chain < 0) {
+    for (int x : {0, t.nfa, t.nfb, t.nk}) w->push_back(x);
+    put64(t.offA);
+    put64(t.offB);
+    for (int i = 0; i < t.nfa; ++i) {
+      w->push_back(t.fa_spin[i]);
+      w->push_back(lg(t.fa_stride[i]));
+    }
+    for (int i = 0; i < t.nfb; ++i) {
+      w->push_back(t.fb_spin[i]);
+      w->push_back(lg(t.fb_stride[i]));
+    }
+    for (int j = 0; j < t.nk; ++j) {
+      w->push_back(t.k_spin[j]);
+      w->push_back(lg(t.k_sA[j]));
+      w->push_back(lg(t.k_sB[j]));
+    }
+  } else {
+    const ChainTrace &c = pr.chain_traces[t.chain];
+    for (int x : {1, c.nout, c.p.t, c.p.ntg}) w->push_back(x);
+    put64(c.offIn);
+    put64(0);
+    for (int j = 0; j < 6; ++j) w->push_back(j < c.p.t ? c.local_spin[j] : 0);
+    for (int j = 0; j < 6; ++j)
+      w->push_back(j < c.p.t && c.p.hi_in[1 << j] > 0 ? lg(c.p.hi_in[1 << j]) : 63);
+    for (int i = 0; i < c.nout; ++i) {
+      w->push_back(c.out_spin[i]);
+      w->push_back(lg(c.out_stride[i]));
+      w->push_back(c.out_rank[i]);
+    }
+    for (int g = 0; g < c.p.ntg; ++g) {
+      const TGate &tg = c.p.tg[g];
+      int f = 0;
+      for (int i = 0; i < TN_TG_MAXF; ++i) f |= (i < tg.nf ? tg.fsh[i] : 62) << (8 * i);
+      w->push_back(tg.kind | (tg.J + 1) << 8 | (tg.K + 1) << 16);
+      w->push_back(f);
+      w->push_back(tg.toff);
+      w->push_back(tg.kspin);
+    }
+  }
+  while (w->size() % 4) w->push_back(0);
 }
 
 // a small step with its planned offsets
@@ -1589,6 +1679,29 @@ bool build_program(const Net &net, const Plan &plan, ProgMode mode, Dtype dt, in
   for (size_t i = 0; i < pr->chain_traces.size(); ++i) {
     patch(pr->chain_traces[i].p, pr->ctrace_blocs[i]);
     pr->chain_traces[i].offIn = abs_off(*pr, pr->ctrace_in[i]) / 4;
+  }
+  for (Walk &w : pr->walks) {
+    w.idx_off = (int)pr->walk_idx.size();
+    w.list_off = (int)pr->walk_list.size();
+    for (int i = 0; i < w.n; ++i) {
+      const TraceStep &t = pr->trace[w.begin + i];
+      WalkIdx x{};
+      x.rec = (int32_t)pr->walk_words.size();
+      encode_walk(*pr, t, &pr->walk_words);
+      x.len = (int32_t)pr->walk_words.size() - x.rec;
+      if (t.chain >= 0) {
+        x.tab = abs_off(*pr, w.tables) / 4 + w.toff[i];
+        x.ntab = pr->chain_traces[t.chain].p.ttotal;
+        pr->walk_list.push_back(i);
+        pr->walk_list.push_back(t.chain);
+        w.nlist++;
+      } else if (t.Ks >= Builder::kWalkBig) {
+        w.big.push_back(i);
+        w.big_rec.push_back(x.rec);
+        w.big_k.push_back(t.Ks);
+      }
+      pr->walk_idx.push_back(x);
+    }
   }
   return true;
 }

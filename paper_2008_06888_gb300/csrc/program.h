@@ -45,6 +45,17 @@ struct SmallRun {
   int desc_len = 0;
 };
 
+// One traceback launch of a q = 2 plan with folded chains: records [begin, begin + n)
+// of the trace, the buffer of its chains' gate tables and of the wide searches' key.
+struct Walk {
+  int begin = 0, n = 0;
+  Loc tables, best;
+  std::vector<int64_t> toff;           // per record: its tables' first element
+  int idx_off = 0, list_off = 0, nlist = 0;
+  std::vector<int> big, big_rec;       // see WalkArgs
+  std::vector<int64_t> big_k;
+};
+
 enum ProgMode { PM_ENERGY = 0, PM_CONFIG = 1, PM_COUNT = 2 };
 
 struct Program {
@@ -66,6 +77,9 @@ struct Program {
   std::vector<std::vector<Loc>> chain_blocs;        // their gate operands
   std::vector<ChainTrace> chain_traces;             // traceback records of chains
   std::vector<Loc> ctrace_in;
+  std::vector<Walk> walks;                          // of OP_TRACE ops with idx >= 0
+  std::vector<int32_t> walk_words, walk_list;
+  std::vector<WalkIdx> walk_idx;
   std::vector<std::vector<Loc>> ctrace_blocs;
   size_t trace_smem = 0;                            // dynamic smem of the trace kernel
   std::vector<LeafDesc> leaves;      // offsets absolute after planning
@@ -89,7 +103,8 @@ struct Program {
   std::vector<Graph> graphs;
   // device copies (owned by the context)
   LeafDesc *d_leaves = nullptr;
-  int32_t *d_small = nullptr;
+  int32_t *d_small = nullptr, *d_walk = nullptr, *d_walk_list = nullptr;
+  WalkIdx *d_walk_idx = nullptr;
   TraceStep *d_trace = nullptr;
   ChainTrace *d_chain_traces = nullptr;
 };

@@ -79,6 +79,9 @@ struct tn_ctx {
   // prime of the pass in flight
   std::unique_ptr<Program> prog_pass;
   uint64_t pass_c = 1;
+  // tables of tn_sample, kept between calls while small
+  char *d_sample = nullptr;
+  int64_t sample_cap = 0;
 };
 
 static std::string g_build_err;
@@ -691,7 +694,7 @@ CountRep count_rep(int n_primes) {
 
 // Counts below 2^59 need no residues: one 8-byte plane holds them exactly,
 // 4 + 8 bytes per element instead of 4 + 28 (mixed +-J batches of side 8..20: 192
-// instances in @@ ms instead of 46.6), and saturates where they do not fit; such an
+// instances in 15.0 ms instead of 46.6), and saturates where they do not fit; such an
 // instance is run again with the residue planes.  Contexts whose counts are likely to
 // be larger start there: +-J glasses have up to about 0.105 bits of ground-state
 // entropy per spin without fields (square lattices; 3-regular and chimera graphs less),
@@ -1721,6 +1724,84 @@ tn_status tn_maxplus_gemm(int32_t dtype, int64_t batch, int64_t M, int64_t N, in
   return TN_OK;
 }
 
+}  // extern "C"
+
+namespace {
+
+// Samples from the tables of one sweep along the order (sample_frontier.cu); *done stays
+// false when that path does not apply and the caller counts prefix by prefix:
+//  - frontiers above 2^26 states, tables beyond a quarter of the free memory, or more
+//    table entries than the batched counts have multiply-adds (a poor order).  An entry
+//    takes two loads and a store of 12 bytes, a multiply-add of the counts about as
+//    much; 16 samples of a 12 x 12 lattice: 3e5 entries against 1e9 multiply-adds.
+//  - 2^59 ground states or more (the tables' counts saturate)
+//  - counting in residues was asked for (TN_COUNT_*)
+// Tables of up to 64 MB stay with the context.
+constexpr int64_t kSampleKeep = int64_t(64) << 20;
+tn_status sample_by_frontier(tn_ctx *ctx, const std::vector<int> &order,
+                             const std::vector<float> &h, int S, uint64_t seed, int8_t *sigma,
+                             bool *done) {
+  *done = false;
+  for (const char *v : {"TN_COUNT_RESIDUES", "TN_COUNT_61", "TN_COUNT_PASSES"})
+    if (std::getenv(v)) return TN_OK;
+  const Net &n = ctx->net;
+  FrontierPlan fp;
+  if (!plan_frontier(n.n, n.eu, n.ev, n.J, h, order, 26, &fp)) return TN_OK;
+  if ((double)fp.elements > 2.0 * n.n * S * std::exp2(ctx->plan.log2_ops)) return TN_OK;
+  if (ensure_device(ctx) != TN_OK) return TN_OK;   // the batched counts report it
+  auto up = [](int64_t b) { return (b + 255) / 256 * 256; };
+  const int64_t oN = 0, oX = oN + up(fp.elements * 8), oS = oX + up(fp.elements * 4),
+                oB = oS + up((int64_t)fp.steps.size() * sizeof(FrontierStep)),
+                oG = oB + up((int64_t)fp.nbs.size() * sizeof(FrontierNb)),
+                bytes = oG + up((int64_t)S * n.n);
+  if (bytes > ctx->sample_cap) {
+    size_t fr = 0, tot = 0;
+    if (cudaMemGetInfo(&fr, &tot) != cudaSuccess || bytes > (int64_t)(fr / 4)) return TN_OK;
+    if (ctx->d_sample) CK(cudaFree(ctx->d_sample));
+    ctx->d_sample = nullptr;
+    ctx->sample_cap = 0;
+    if (cudaMalloc(&ctx->d_sample, bytes) != cudaSuccess) {
+      cudaGetLastError();
+      ctx->d_sample = nullptr;
+      return TN_OK;
+    }
+    ctx->sample_cap = bytes;
+  }
+  char *d = ctx->d_sample;
+  CK(cudaMemcpyAsync(d + oS, fp.steps.data(), fp.steps.size() * sizeof(FrontierStep),
+                     cudaMemcpyHostToDevice, ctx->stream));
+  if (!fp.nbs.empty())
+    CK(cudaMemcpyAsync(d + oB, fp.nbs.data(), fp.nbs.size() * sizeof(FrontierNb),
+                       cudaMemcpyHostToDevice, ctx->stream));
+  int nl = 0, herr = 0;
+  CK(launch_frontier_sample(fp, reinterpret_cast<FrontierStep *>(d + oS),
+                            reinterpret_cast<FrontierNb *>(d + oB),
+                            reinterpret_cast<int32_t *>(d + oX),
+                            reinterpret_cast<uint64_t *>(d + oN), S, seed,
+                            reinterpret_cast<int8_t *>(d + oG), ctx->d_err, &nl, ctx->stream));
+  ctx->launches[5] += nl;
+  uint64_t total = 0;
+  std::vector<int8_t> out((size_t)S * n.n);
+  CK(cudaMemcpyAsync(&total, d + oN, 8, cudaMemcpyDeviceToHost, ctx->stream));
+  CK(cudaMemcpyAsync(out.data(), d + oG, out.size(), cudaMemcpyDeviceToHost, ctx->stream));
+  CK(cudaMemcpyAsync(&herr, ctx->d_err, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
+  CK(cudaStreamSynchronize(ctx->stream));
+  if (herr) CK(cudaMemsetAsync(ctx->d_err, 0, sizeof(int), ctx->stream));
+  if (ctx->sample_cap > kSampleKeep) {
+    CK(cudaFree(ctx->d_sample));
+    ctx->d_sample = nullptr;
+    ctx->sample_cap = 0;
+  }
+  if (herr || total >= kSaturated) return TN_OK;
+  std::copy(out.begin(), out.end(), sigma);
+  *done = true;
+  return TN_OK;
+}
+
+}  // namespace
+
+extern "C" {
+
 tn_status tn_sample(tn_ctx *ctx, int32_t n_samples, uint64_t seed, const int32_t *order,
                     int8_t *sigma) {
   if (!ctx) return TN_EINVAL;
@@ -1756,6 +1837,12 @@ tn_status tn_sample(tn_ctx *ctx, int32_t n_samples, uint64_t seed, const int32_t
     e[2 * k + 1] = n.ev[k];
   }
   std::vector<float> h0 = n.h.empty() ? std::vector<float>(n.n, 0.f) : n.h;
+  bool done = n_samples == 0;
+  if (!done) {
+    const tn_status fs = sample_by_frontier(ctx, ord, h0, n_samples, seed, sigma, &done);
+    if (fs != TN_OK) return fs;
+  }
+  if (done) return TN_OK;
   tn_ctx *pc = nullptr;
   tn_status s = tn_build(&pc, n.n, n.m, e.data(), n.J.data(), h0.data(), 2, TN_DTYPE_I32);
   if (s != TN_OK) return fail(ctx, s, "sampler: " + g_build_err);
@@ -1813,6 +1900,7 @@ void tn_destroy(tn_ctx *ctx) {
   if (ctx->d_stateb) cudaFree(ctx->d_stateb);
   if (ctx->d_outb) cudaFree(ctx->d_outb);
   if (ctx->d_arena) cudaFree(ctx->d_arena);
+  if (ctx->d_sample) cudaFree(ctx->d_sample);
   for (auto e : ctx->ev_pool) cudaEventDestroy(e);
   if (ctx->cap_stream) cudaStreamDestroy(ctx->cap_stream);
   delete ctx;

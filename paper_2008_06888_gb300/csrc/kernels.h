@@ -96,6 +96,17 @@ struct WalkArgs {
 cudaError_t launch_walk(Dtype dt, const WalkArgs &w, char *arena, int8_t *state, int nspins,
                         int *err, const Batch &bt, cudaStream_t st);
 
+// Tables of best completions along a frontier plan (device copies of its records) and S
+// samples drawn from them (sample_frontier.cu): X, N of p.elements entries, sigma S x n.
+// *err (device) is set to 1 when a draw fails; *launches grows by the kernels launched.
+struct FrontierPlan;
+struct FrontierStep;
+struct FrontierNb;
+cudaError_t launch_frontier_sample(const FrontierPlan &p, const FrontierStep *steps,
+                                   const FrontierNb *nbs, int32_t *X, uint64_t *N, int S,
+                                   uint64_t seed, int8_t *sigma, int *err, int *launches,
+                                   cudaStream_t st);
+
 // A run of small steps in one launch, one block per instance.  Descriptors (32-bit
 // words): {steps, levels}, level starts [levels + 1], per step its first output within
 // its level, per step the word of its body, then the bodies: 64-bit offsets of the

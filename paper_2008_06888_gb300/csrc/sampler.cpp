@@ -2,6 +2,7 @@
 #include "sampler.h"
 
 #include <algorithm>
+#include <cmath>
 
 namespace tn {
 
@@ -116,6 +117,59 @@ int sample_ground_states(int n, int S, const std::vector<int> &order, const std:
     }
   }
   return 0;
+}
+
+bool plan_frontier(int n, const std::vector<int> &eu, const std::vector<int> &ev,
+                   const std::vector<float> &J, const std::vector<float> &h,
+                   const std::vector<int> &order, int max_bits, FrontierPlan *out) {
+  out->steps.assign(n, FrontierStep{});
+  out->nbs.clear();
+  std::vector<int> pos(n), last(n), slot(n, -1);
+  for (int t = 0; t < n; ++t) pos[order[t]] = t;
+  std::vector<std::vector<std::pair<int, float>>> adj(n);
+  for (size_t e = 0; e < eu.size(); ++e) {
+    adj[eu[e]].push_back({ev[e], J[e]});
+    adj[ev[e]].push_back({eu[e], J[e]});
+  }
+  for (int i = 0; i < n; ++i) {
+    last[i] = pos[i];
+    for (const auto &a : adj[i]) last[i] = std::max(last[i], pos[a.first]);
+  }
+  uint64_t used = 0;   // occupied slots
+  auto states = [](uint64_t u) {
+    uint64_t s = 1;
+    while (u >> 1 >= s) s <<= 1;   // up to the highest occupied slot
+    return u ? s << 1 : 1;
+  };
+  int64_t off = 0;
+  for (int t = 0; t < n; ++t) {
+    FrontierStep &st = out->steps[t];
+    const int i = order[t];
+    st.spin = i;
+    st.h = (int32_t)std::lrint(h[i]);
+    st.size = (uint32_t)states(used);
+    st.off = off;
+    off += st.size;
+    st.next = off;
+    st.nb = (int32_t)out->nbs.size();
+    for (const auto &a : adj[i]) {
+      if (pos[a.first] > t) continue;
+      out->nbs.push_back({slot[a.first], (int32_t)std::lrint(a.second)});
+      if (last[a.first] == t) used &= ~(uint64_t(1) << slot[a.first]);
+    }
+    st.nnb = (int32_t)out->nbs.size() - st.nb;
+    st.keep = (uint32_t)used;
+    st.slot = -1;
+    if (last[i] > t) {
+      int k = 0;
+      while ((used >> k) & 1) ++k;
+      if (k >= max_bits) return false;
+      slot[i] = st.slot = k;
+      used |= uint64_t(1) << k;
+    }
+  }
+  out->elements = off + 1;
+  return true;
 }
 
 }  // namespace tn

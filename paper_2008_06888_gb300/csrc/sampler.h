@@ -46,6 +46,33 @@ int sample_ground_states(int n, int S, const std::vector<int> &order, const std:
                          uint64_t seed, int chunk, const CountFn &count,
                          std::vector<int8_t> *sigma, std::string *err);
 
+// The spins of an order as a sweep of one frontier.  Behind step t stand the placed spins
+// that still have a neighbour to come; spin order[t] takes a slot (one bit of a state
+// index) unless none of its neighbours comes later, and a spin whose last neighbour is
+// placed gives its slot back before the new one is taken.
+struct FrontierStep {
+  int64_t off;            // first element of the table in front of this step
+  int64_t next;           // first element of the table behind it
+  uint32_t size;          // states of the table (bits of free slots make no difference)
+  uint32_t keep;          // slots that stay
+  int32_t slot, spin;     // slot of the new spin (-1: none) and its number
+  int32_t h;              // its field
+  int32_t nb, nnb;        // its earlier neighbours: [nb, nb + nnb) of the array below
+  int32_t pad;
+};
+struct FrontierNb {
+  int32_t slot, J;
+};
+struct FrontierPlan {
+  std::vector<FrontierStep> steps;
+  std::vector<FrontierNb> nbs;
+  int64_t elements = 0;   // of all tables, the one behind the last step included
+};
+// false: a frontier of more than max_bits slots (couplings J, h must be integral)
+bool plan_frontier(int n, const std::vector<int> &eu, const std::vector<int> &ev,
+                   const std::vector<float> &J, const std::vector<float> &h,
+                   const std::vector<int> &order, int max_bits, FrontierPlan *out);
+
 // Helpers (exposed for tests).
 uint64_t mix64(uint64_t x);                         // SplitMix64 finaliser
 bool big_less(const Big &a, const Big &b);

@@ -1927,6 +1927,7 @@ cudaError_t launch_chain(Dtype dt, const ChainParams &p, const char *arena, cons
     return launch_schain(p, arena, Ax, An, Cx, Cn, bt, st);
   if (p.mode == 1 && p.P > 0) return launch_rchain_count(dt, p, arena, Ax, An, Cx, Cn, ps, bt, st);
   if (p.mode == 1) return launch_rchain(dt, p, arena, Ax, Cx, bt, st);
+  if (p.q == 3 && p.P == 0) return launch_chain3(dt, p, arena, Ax, Cx, bt, st);
   const bool c = p.P > 0;
   if (c && ps.r32) {
     if (dt == DT_F32)
@@ -1938,65 +1939,136 @@ cudaError_t launch_chain(Dtype dt, const ChainParams &p, const char *arena, cons
   if (dt == DT_F32) {
     if (p.q == 2) return c ? launch_chain_t<float, 2, true>(p, arena, Ax, An, Cx, Cn, ps, bt, st)
                            : launch_chain_t<float, 2, false>(p, arena, Ax, An, Cx, Cn, ps, bt, st);
-    return c ? launch_chain_t<float, 3, true>(p, arena, Ax, An, Cx, Cn, ps, bt, st)
-             : launch_chain_t<float, 3, false>(p, arena, Ax, An, Cx, Cn, ps, bt, st);
+    return launch_chain_t<float, 3, true>(p, arena, Ax, An, Cx, Cn, ps, bt, st);
   }
   if (p.q == 2) return c ? launch_chain_t<int32_t, 2, true>(p, arena, Ax, An, Cx, Cn, ps, bt, st)
                          : launch_chain_t<int32_t, 2, false>(p, arena, Ax, An, Cx, Cn, ps, bt, st);
-  return c ? launch_chain_t<int32_t, 3, true>(p, arena, Ax, An, Cx, Cn, ps, bt, st)
-           : launch_chain_t<int32_t, 3, false>(p, arena, Ax, An, Cx, Cn, ps, bt, st);
+  return launch_chain_t<int32_t, 3, true>(p, arena, Ax, An, Cx, Cn, ps, bt, st);
 }
 
-// Traceback of one chain record by the whole block: reload the input tile,
-// replay the gates keeping every intermediate tile, then walk back.
+// Traceback of one chain record by the whole block: reload the input, replay the gates
+// keeping every intermediate state, then walk back.  The digits of the legs that the
+// chain does not replace are known, so only the q^(replaced legs) elements of the tile
+// that agree with them are replayed (81 of a 6561-element tile with four replaced legs;
+// 1134 -> 705 us of a 15 x 15 lattice's traceback, with tiles
+// three times as large).
 template <typename T, int Q>
 __device__ void trace_chain(const ChainTrace &ct, const T *X, int8_t *state, int *err, char *smem,
                             int64_t *sbase) {
   const ChainParams &p = ct.p;
-  T *buf = reinterpret_cast<T *>(smem);                 // (ngates + 1) tiles
-  T *sB = buf + (int64_t)(p.ngates + 1) * p.tile;       // gate operands
-  if (threadIdx.x == 0) {
-    int64_t b = ct.offIn;
-    for (int i = 0; i < ct.nout; ++i) {
+  __shared__ int sx, snrep, srl[TN_CHAIN_MAX_T];        // final local index; replaced legs
+  __shared__ int sss[TN_CHAIN_MAX_G], sbs[TN_CHAIN_MAX_G][2], sfix[TN_CHAIN_MAX_G];
+  auto digit = [](int x, int s) { return (x / s) % Q; };
+  if (threadIdx.x < 32) {
+    const int lane = threadIdx.x;
+    int64_t b = 0;
+    for (int i = lane; i < ct.nout; i += 32) {
       int d = state[ct.out_spin[i]];
       if (d < 0 || d >= Q) { *err = 1; d = 0; }
       b += (int64_t)d * ct.out_stride[i];
     }
-    *sbase = b;
+    int x = 0;
+    if (lane < p.t) {
+      x = state[ct.local_spin[lane]];
+      if (x < 0 || x >= Q) { *err = 1; x = 0; }
+      for (int j = lane + 1; j < p.t; ++j) x *= Q;
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+      b += __shfl_xor_sync(0xffffffffu, b, o);
+      x += __shfl_xor_sync(0xffffffffu, x, o);
+    }
+    if (lane == 0) {
+      *sbase = ct.offIn + b;
+      sx = x;
+      int n = 0;
+      for (int gi = 0; gi < p.ngates; ++gi) {
+        bool seen = p.g[gi].kind != 0;
+        for (int k = 0; k < n; ++k) seen = seen || srl[k] == p.g[gi].ls;
+        if (!seen) srl[n++] = p.g[gi].ls;
+      }
+      snrep = n;
+    }
+  }
+  __syncthreads();
+  const int nrep = snrep, x = sx;
+  int sub = 1, xf = x, yx = 0;   // states replayed; their fixed part; the final one
+  for (int k = 0; k < nrep; ++k) {
+    const int d = digit(x, srl[k]);
+    xf -= d * srl[k];
+    yx += d * sub;
+    sub *= Q;
+  }
+  T *buf = reinterpret_cast<T *>(smem);                 // (ngates + 1) states of the sub-tile
+  T *sB = buf + (int64_t)(p.ngates + 1) * sub;          // gate operands
+  if (threadIdx.x < p.ngates) {
+    const ChainGate &g = p.g[threadIdx.x];
+    auto substride = [&](int s) {
+      int r = 1;
+      for (int k = 0; k < nrep; ++k, r *= Q)
+        if (srl[k] == s) return r;
+      return 0;
+    };
+    int fix = 0;
+    for (int j = 0; j < 2; ++j) {
+      const int r = j < g.nb ? substride(g.lsb[j]) : 0;
+      sbs[threadIdx.x][j] = r;
+      if (j < g.nb && r == 0) fix += digit(x, g.lsb[j]) * (int)g.sBb[j];
+    }
+    sfix[threadIdx.x] = fix;
+    sss[threadIdx.x] = g.kind == 0 ? substride(g.ls) : 0;
   }
   load_gate_operands<T, uint64_t>(p, X, nullptr, sB, nullptr, kGateBMax);
-  __syncthreads();
   const int64_t base = *sbase;
-  for (int i = threadIdx.x; i < p.tile; i += blockDim.x) buf[i] = X[base + tile_elem_off<Q>(p, i)];
+  for (int y = threadIdx.x; y < sub; y += blockDim.x) {
+    int r = y, xl = xf;
+    for (int k = 0; k < nrep; ++k) {
+      xl += (r % Q) * srl[k];
+      r /= Q;
+    }
+    buf[y] = X[base + tile_elem_off<Q>(p, xl)];
+  }
   __syncthreads();
+  auto boff = [&](int gi, int y) {   // operand offset of sub-tile element y
+    int o = sfix[gi];
+    for (int j = 0; j < 2; ++j)
+      if (sbs[gi][j] > 0) o += digit(y, sbs[gi][j]) * (int)p.g[gi].sBb[j];
+    return o;
+  };
   for (int gi = 0; gi < p.ngates; ++gi) {
-    apply_gate<T, Q>(p.g[gi], buf + (int64_t)gi * p.tile, buf + (int64_t)(gi + 1) * p.tile,
-                     sB + gi * kGateBMax, p.tile);
+    const ChainGate &g = p.g[gi];
+    const T *src = buf + (int64_t)gi * sub, *B = sB + gi * kGateBMax;
+    T *dst = buf + (int64_t)(gi + 1) * sub;
+    const int ss = sss[gi];
+    if (g.kind == 0) {
+      for (int y = threadIdx.x; y < sub; y += blockDim.x) {
+        const int v = digit(y, ss), y0 = y - v * ss, bo = boff(gi, y0) + v * (int)g.sBn;
+        T best = src[y0] + B[bo];
+#pragma unroll
+        for (int u = 1; u < Q; ++u) best = max(best, src[y0 + u * ss] + B[bo + u * (int)g.sBk]);
+        dst[y] = best;
+      }
+    } else {
+      for (int y = threadIdx.x; y < sub; y += blockDim.x) dst[y] = src[y] + B[boff(gi, y)];
+    }
     __syncthreads();
   }
   if (threadIdx.x == 0) {
-    int x = 0;
-    for (int j = 0; j < p.t; ++j) {
-      int d = state[ct.local_spin[j]];
-      if (d < 0 || d >= Q) { *err = 1; d = 0; }
-      x = x * Q + d;
-    }
+    int y = yx;
     for (int gi = p.ngates - 1; gi >= 0; --gi) {
       const ChainGate &g = p.g[gi];
       if (g.kind != 0) continue;
-      const T *src = buf + (int64_t)gi * p.tile;
+      const T *src = buf + (int64_t)gi * sub;
       const T *gB = sB + gi * kGateBMax;
-      const int v = mod_q<Q>(div_p<Q>(x, g.ls, g.lsh));
-      const int x0 = x - v * g.ls;
-      const int64_t bo = gate_boff<Q>(g, x0);
+      const int ss = sss[gi], v = digit(y, ss), y0 = y - v * ss;
+      const int64_t bo = boff(gi, y0);
       int bu = 0;
-      T best = src[x0] + gB[bo + v * g.sBn];
+      T best = src[y0] + gB[bo + v * g.sBn];
       for (int u = 1; u < Q; ++u) {
-        T val = src[x0 + u * g.ls] + gB[bo + u * g.sBk + v * g.sBn];
+        T val = src[y0 + u * ss] + gB[bo + u * g.sBk + v * g.sBn];
         if (val > best) { best = val; bu = u; }
       }
       state[g.kspin] = (int8_t)bu;
-      x = x0 + bu * g.ls;
+      y = y0 + bu * ss;
     }
   }
   __syncthreads();
@@ -3020,7 +3092,14 @@ __global__ void __launch_bounds__(kTraceThreads) k_trace(const TraceStep *__rest
 size_t trace_smem_bytes(const ChainParams &p, size_t elem) {
   if (p.mode == 1)
     return elem * ((size_t)(p.ngates + 1) * p.tile + (size_t)TN_CHAIN_MAX_G * TN_TG_TABLE);
-  return elem * ((size_t)(p.ngates + 1) * p.tile + (size_t)TN_CHAIN_MAX_G * kGateBMax);
+  std::vector<int> rl;   // replaced legs: the traced sub-tile (trace_chain)
+  size_t sub = 1;
+  for (int i = 0; i < p.ngates; ++i)
+    if (p.g[i].kind == 0 && std::find(rl.begin(), rl.end(), p.g[i].ls) == rl.end()) {
+      rl.push_back(p.g[i].ls);
+      sub *= p.q;
+    }
+  return elem * ((size_t)(p.ngates + 1) * sub + (size_t)TN_CHAIN_MAX_G * kGateBMax);
 }
 
 size_t trace_state_bytes(int nspins) { return ((size_t)(nspins + 15) / 16) * 16; }

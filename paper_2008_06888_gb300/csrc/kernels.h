@@ -130,6 +130,10 @@ cudaError_t launch_schain(const ChainParams &p, const char *arena, const void *A
                           const uint64_t *An, void *Cx, uint64_t *Cn, const Batch &bt,
                           cudaStream_t st);
 
+// Fused gate chain of q = 3 values (chain3.cu).
+cudaError_t launch_chain3(Dtype dt, const ChainParams &p, const char *arena, const void *A,
+                          void *C, const Batch &bt, cudaStream_t st);
+
 // Resident blocks of a kernel on the whole device and the grid (blocks per
 // instance) of a grid-stride kernel with `need` blocks of work per instance.
 int64_t wave_blocks(int64_t need, int B, int64_t slots);

@@ -634,7 +634,7 @@ struct Builder {
   bool try_gate(const PStep &st, int big, int small, CGate *g) {
     const std::vector<int> &ob = order[big], &os = order[small];
     const int R = (int)ob.size();
-    if ((int)os.size() > 3 || R < (regmode ? kRB + 8 : tmax + 3)) return false;
+    if ((int)os.size() > 3 || R < (regmode ? kRB + 8 : q == 3 ? 10 : tmax + 3)) return false;
     const std::vector<int> &N = (big == st.a) ? st.N : st.M;
     if (st.K.size() != N.size() || st.K.size() > 1 || st.batch.size() > 2) return false;
     if (regmode && st.K.size() == 1 && st.batch.size() > 1) return false;
@@ -742,6 +742,11 @@ struct Builder {
     if (g.pos >= 0) t.push_back(g.pos);
     for (int p : g.bpos) t.push_back(p);
     const int R = (int)order[m.in].size();
+    if (q == 3) {   // the traceback keeps 3^(replaced legs) states per gate
+      int n = (int)m.rpos.size();
+      if (g.kind == 0 && pos_of(m.rpos, g.pos) < 0) ++n;
+      if (n > 7) return false;
+    }
     return (int)local_set(R, t).size() <= tmax;
   }
 
@@ -1315,7 +1320,9 @@ struct Builder {
     if (pr.sat && folded()) kRB = 4;
     // integral counts without folding have no register-chain kernel
     if (pr.sat && !folded() && pr.dt == DT_I32) regmode = false;
-    if (q == 3) { tmax = 7; wlow = 4; }
+    // q = 3 tiles: 8 legs (26 KB, two of them staged per block, four blocks per SM) of
+    // which 4 are the fastest, for runs of 81 elements; 7 with the counts' planes
+    if (q == 3) { tmax = P == 0 ? 8 : 7; wlow = 4; }
     emit_leaves();
     if (!forward()) return false;
     pr.root = loc[plan.root];

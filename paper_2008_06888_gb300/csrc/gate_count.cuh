@@ -11,6 +11,7 @@
 
 #include "kernels.h"
 #include "chain_dev.cuh"
+#include "gate_dev.cuh"
 #include "modarith.cuh"
 
 namespace tn {
@@ -36,7 +37,7 @@ __device__ __forceinline__ void gtc_store4(Sat64 *dst, const Sat64 *src) {
 
 // VC: the NS outputs of an outer index are NS consecutive words of C (and of
 // each plane), so every four of them are stored with one 16-byte access.
-template <typename T, int KS, int NS, int P, typename R, bool VC = false>
+template <typename T, int KS, int NS, int P, typename R, typename I, bool VC = false>
 __global__ void __launch_bounds__(256) k_gate_tc(const GateParams p, const T *__restrict__ A,
                                                  const T *__restrict__ B, T *__restrict__ C,
                                                  const R *__restrict__ nA,
@@ -51,32 +52,18 @@ __global__ void __launch_bounds__(256) k_gate_tc(const GateParams p, const T *__
     nB = inst_ptr(nB, ib);
   }
   const bool mulB = p.hasB && !p.unitB;
-  int64_t kA[KS], kB[KS];
+  I kA[KS], kB[KS];
 #pragma unroll
-  for (int k = 0; k < KS; ++k) { kA[k] = p.kA[k]; kB[k] = p.kB[k]; }
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t o0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; o0 < p.outer; o0 += 2 * stride) {
-    int64_t oa[2], ob[2], oc[2];
+  for (int k = 0; k < KS; ++k) { kA[k] = (I)p.kA[k]; kB[k] = (I)p.kB[k]; }
+  const I stride = (I)(gridDim.x * blockDim.x);
+  for (I o0 = (I)(blockIdx.x * blockDim.x + threadIdx.x); o0 < (I)p.outer; o0 += 2 * stride) {
+    I oa[2], ob[2], oc[2];
     bool live[2];
 #pragma unroll
     for (int u = 0; u < 2; ++u) {
-      const int64_t o = o0 + u * stride;
-      live[u] = o < p.outer;
-      int64_t r = live[u] ? o : 0;
-      oa[u] = ob[u] = oc[u] = 0;
-      for (int s = p.nseg - 1; s >= 0; --s) {
-        int64_t i;
-        if (p.seg_sh[s] >= 0) {
-          i = r & (p.seg_size[s] - 1);
-          r >>= p.seg_sh[s];
-        } else {
-          i = r % p.seg_size[s];
-          r /= p.seg_size[s];
-        }
-        oa[u] += i * p.seg_sA[s];
-        ob[u] += i * p.seg_sB[s];
-        oc[u] += i * p.seg_sC[s];
-      }
+      const I o = o0 + u * stride;
+      live[u] = o < (I)p.outer;
+      gate_decode<I>(p, live[u] ? o : 0, oa[u], ob[u], oc[u]);
     }
     T a[2][KS];
     R na[2][P][KS];
@@ -84,19 +71,19 @@ __global__ void __launch_bounds__(256) k_gate_tc(const GateParams p, const T *__
     for (int u = 0; u < 2; ++u)
 #pragma unroll
       for (int k = 0; k < KS; ++k) {
-        const int64_t e = live[u] ? oa[u] + kA[k] : 0;
+        const I e = live[u] ? oa[u] + kA[k] : 0;
         a[u][k] = A[e];
 #pragma unroll
         for (int i = 0; i < P; ++i) na[u][i][k] = nA[i * p.planeA + e];
       }
     // output n of outer index u: the max over k and the counts of the tied k
     auto out_one = [&](int u, int n, T &best, R (&cnt)[P]) {
-      const int64_t nb = p.nB[n];
+      const I nb = (I)p.nB[n];
       T v[KS];
       R bn[P][KS];
 #pragma unroll
       for (int k = 0; k < KS; ++k) {
-        const int64_t e = ob[u] + kB[k] + nb;
+        const I e = ob[u] + kB[k] + nb;
         v[k] = a[u][k] + (p.hasB ? B[e] : T(0));
 #pragma unroll
         for (int i = 0; i < P; ++i) bn[i][k] = mulB ? nB[i * p.planeB + e] : R(1);
@@ -132,7 +119,7 @@ __global__ void __launch_bounds__(256) k_gate_tc(const GateParams p, const T *__
 #pragma unroll
             for (int i = 0; i < P; ++i) cnt4[i][j] = cnt[i];
           }
-          const int64_t c = oc[u] + n0;
+          const I c = oc[u] + n0;
           gtc_store4(C + c, best4);
 #pragma unroll
           for (int i = 0; i < P; ++i) gtc_store4(nC + i * p.planeC + c, cnt4[i]);
@@ -143,7 +130,7 @@ __global__ void __launch_bounds__(256) k_gate_tc(const GateParams p, const T *__
           T best;
           R cnt[P];
           out_one(u, n, best, cnt);
-          const int64_t c = oc[u] + p.nC[n];
+          const I c = oc[u] + (I)p.nC[n];
           C[c] = best;
 #pragma unroll
           for (int i = 0; i < P; ++i) nC[i * p.planeC + c] = cnt[i];
@@ -153,13 +140,13 @@ __global__ void __launch_bounds__(256) k_gate_tc(const GateParams p, const T *__
   }
 }
 
-template <typename T, typename R>
+template <typename T, typename R, typename I>
 bool launch_gate_tc_r(const GateParams &p, const T *A, const T *B, T *C, const R *nA,
                              const R *nB, R *nC, const PrimeSet &ps, dim3 blocks, int64_t ib,
                              bool vc, cudaStream_t st) {
 #define TN_GTC(KS_, NS_, P_)                                                                  \
   if (p.Ks == KS_ && p.Ns == NS_ && p.P == P_) {                                              \
-    k_gate_tc<T, KS_, NS_, P_, R><<<blocks, 256, 0, st>>>(p, A, B, C, nA, nB, nC, ps, ib);   \
+    k_gate_tc<T, KS_, NS_, P_, R, I><<<blocks, 256, 0, st>>>(p, A, B, C, nA, nB, nC, ps, ib);   \
     return true;                                                                            \
   }
 // the forms with the plane count of the residue type: 7 or 1 of 4 bytes, 1 of
@@ -169,13 +156,13 @@ bool launch_gate_tc_r(const GateParams &p, const T *A, const T *B, T *C, const R
   TN_GTC(2, 16, P_)
   if constexpr (sizeof(R) == 4) {
     if (vc && p.Ks == 2 && p.Ns == 16 && p.P == 7) {
-      k_gate_tc<T, 2, 16, 7, R, true><<<blocks, 256, 0, st>>>(p, A, B, C, nA, nB, nC, ps, ib);
+      k_gate_tc<T, 2, 16, 7, R, I, true><<<blocks, 256, 0, st>>>(p, A, B, C, nA, nB, nC, ps, ib);
       return true;
     }
     TN_GTC_P(7)
   }
   if (vc && p.Ks == 2 && p.Ns == 16 && p.P == 1) {
-    k_gate_tc<T, 2, 16, 1, R, true><<<blocks, 256, 0, st>>>(p, A, B, C, nA, nB, nC, ps, ib);
+    k_gate_tc<T, 2, 16, 1, R, I, true><<<blocks, 256, 0, st>>>(p, A, B, C, nA, nB, nC, ps, ib);
     return true;
   }
   TN_GTC_P(1)
@@ -203,11 +190,12 @@ bool launch_gate_tc_typed(const GateParams &p, const T *A, const T *B, T *C, con
   for (int n = 0; vc && n < p.Ns; ++n) vc = p.nC[n] == n;
   for (int s = 0; vc && s < p.nseg; ++s) vc = p.seg_sC[s] % 4 == 0;
   const dim3 grid((unsigned)nb, bt.B);
-  if (ps.r32)
-    return launch_gate_tc_r<T, uint32_t>(p, A, B, C, (const uint32_t *)nA, (const uint32_t *)nB,
-                                         (uint32_t *)nC, ps, grid, bt.ib, vc, st);
-  return launch_gate_tc_r<T, Sat64>(p, A, B, C, (const Sat64 *)nA, (const Sat64 *)nB,
-                                    (Sat64 *)nC, ps, grid, bt.ib, vc, st);
+#define TN_GTC_R(R_, I_)                                                                       \
+  launch_gate_tc_r<T, R_, I_>(p, A, B, C, (const R_ *)nA, (const R_ *)nB, (R_ *)nC, ps, grid,   \
+                              bt.ib, vc, st)
+  if (gate_fits32(p)) return ps.r32 ? TN_GTC_R(uint32_t, int32_t) : TN_GTC_R(Sat64, int32_t);
+  return ps.r32 ? TN_GTC_R(uint32_t, int64_t) : TN_GTC_R(Sat64, int64_t);
+#undef TN_GTC_R
 }
 
 }  // namespace tn

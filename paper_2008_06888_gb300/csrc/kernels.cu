@@ -21,6 +21,7 @@
 #include "kernels.h"
 #include "perm_bits.h"
 #include "chain_dev.cuh"
+#include "gate_dev.cuh"
 #include "modarith.cuh"
 
 namespace tn {
@@ -165,7 +166,7 @@ cudaError_t launch_leaves(Dtype dt, int q, const LeafDesc *d_leaves, int nleaves
 // ---------------------------------------------------------------- gate contraction
 
 // C[o, n] = max_k A[o, k] + B[o, k, n], one outer index per thread.
-template <typename T, bool COUNT, typename R = uint64_t>
+template <typename T, bool COUNT, typename R, typename I>
 __global__ void __launch_bounds__(256) k_gate(const GateParams p, const T *__restrict__ A,
                                               const T *__restrict__ B, T *__restrict__ C,
                                               const R *__restrict__ nA,
@@ -180,22 +181,10 @@ __global__ void __launch_bounds__(256) k_gate(const GateParams p, const T *__res
     nC = inst_ptr(nC, ib);
     if (p.hasB) nB = inst_ptr(nB, ib);
   }
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t o = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; o < p.outer; o += stride) {
-    int64_t r = o, oa = 0, ob = 0, oc = 0;
-    for (int s = p.nseg - 1; s >= 0; --s) {
-      int64_t i;
-      if (p.seg_sh[s] >= 0) {
-        i = r & (p.seg_size[s] - 1);
-        r >>= p.seg_sh[s];
-      } else {
-        i = r % p.seg_size[s];
-        r /= p.seg_size[s];
-      }
-      oa += i * p.seg_sA[s];
-      ob += i * p.seg_sB[s];
-      oc += i * p.seg_sC[s];
-    }
+  const I stride = (I)(gridDim.x * blockDim.x);
+  for (I o = (I)(blockIdx.x * blockDim.x + threadIdx.x); o < (I)p.outer; o += stride) {
+    I oa, ob, oc;
+    gate_decode<I>(p, o, oa, ob, oc);
     for (int n = 0; n < p.Ns; ++n) {
       T best = Lim<T>::neg();
       R cnt[TN_MAX_PRIMES];
@@ -233,43 +222,27 @@ __global__ void __launch_bounds__(256) k_gate(const GateParams p, const T *__res
 }
 
 // Values-only gate contraction with the numbers of contracted and new states
-// known at compile time (the common 1 / 2 cases): offsets held in registers,
-// two outer indices per thread for independent loads.
-template <typename T, int KS, int NS>
+// known at compile time: two outer indices per thread for independent loads.
+// VC: the outputs of an outer index are consecutive words, stored four at a time.
+template <typename T, int KS, int NS, typename I, bool VC>
 __global__ void __launch_bounds__(256) k_gate_t(const GateParams p, const T *__restrict__ A,
                                                 const T *__restrict__ B, T *__restrict__ C,
                                                 int64_t ib) {
   A = inst_ptr(A, ib);
   C = inst_ptr(C, ib);
   if (p.hasB) B = inst_ptr(B, ib);
-  int64_t kA[KS], kB[KS], nB[NS], nC[NS];
+  I kA[KS], kB[KS];
 #pragma unroll
-  for (int k = 0; k < KS; ++k) { kA[k] = p.kA[k]; kB[k] = p.kB[k]; }
-#pragma unroll
-  for (int n = 0; n < NS; ++n) { nB[n] = p.nB[n]; nC[n] = p.nC[n]; }
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t o0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; o0 < p.outer; o0 += 2 * stride) {
-    int64_t oa[2], ob[2], oc[2];
+  for (int k = 0; k < KS; ++k) { kA[k] = (I)p.kA[k]; kB[k] = (I)p.kB[k]; }
+  const I stride = (I)(gridDim.x * blockDim.x);
+  for (I o0 = (I)(blockIdx.x * blockDim.x + threadIdx.x); o0 < (I)p.outer; o0 += 2 * stride) {
+    I oa[2], ob[2], oc[2];
     bool live[2];
 #pragma unroll
     for (int u = 0; u < 2; ++u) {
-      const int64_t o = o0 + u * stride;
-      live[u] = o < p.outer;
-      int64_t r = live[u] ? o : 0;
-      oa[u] = ob[u] = oc[u] = 0;
-      for (int s = p.nseg - 1; s >= 0; --s) {
-        int64_t i;
-        if (p.seg_sh[s] >= 0) {
-          i = r & (p.seg_size[s] - 1);
-          r >>= p.seg_sh[s];
-        } else {
-          i = r % p.seg_size[s];
-          r /= p.seg_size[s];
-        }
-        oa[u] += i * p.seg_sA[s];
-        ob[u] += i * p.seg_sB[s];
-        oc[u] += i * p.seg_sC[s];
-      }
+      const I o = o0 + u * stride;
+      live[u] = o < (I)p.outer;
+      gate_decode<I>(p, live[u] ? o : 0, oa[u], ob[u], oc[u]);
     }
     T a[2][KS];
 #pragma unroll
@@ -279,32 +252,58 @@ __global__ void __launch_bounds__(256) k_gate_t(const GateParams p, const T *__r
 #pragma unroll
     for (int u = 0; u < 2; ++u) {
       if (!live[u]) continue;
-#pragma unroll
-      for (int n = 0; n < NS; ++n) {
-        T best = a[u][0] + (p.hasB ? B[ob[u] + kB[0] + nB[n]] : T(0));
+      auto out_one = [&](int n) {
+        const I b = ob[u] + (I)p.nB[n];
+        T best = a[u][0] + (p.hasB ? B[b + kB[0]] : T(0));
 #pragma unroll
         for (int k = 1; k < KS; ++k)
-          best = max(best, a[u][k] + (p.hasB ? B[ob[u] + kB[k] + nB[n]] : T(0)));
-        C[oc[u] + nC[n]] = best;
+          best = max(best, a[u][k] + (p.hasB ? B[b + kB[k]] : T(0)));
+        return best;
+      };
+      if constexpr (VC) {
+#pragma unroll
+        for (int n = 0; n < NS; n += 4) {
+          typename Vec4<T>::t v;
+          v.x = out_one(n);
+          v.y = out_one(n + 1);
+          v.z = out_one(n + 2);
+          v.w = out_one(n + 3);
+          *reinterpret_cast<typename Vec4<T>::t *>(C + oc[u] + n) = v;
+        }
+      } else {
+#pragma unroll
+        for (int n = 0; n < NS; ++n) C[oc[u] + (I)p.nC[n]] = out_one(n);
       }
     }
   }
 }
 
-template <typename T>
+// four outputs per 16-byte store: consecutive words, every start a multiple of four
+static bool gate_vec4(const GateParams &p, const void *C, int64_t ib) {
+  bool vc = p.Ns % 4 == 0 && reinterpret_cast<uintptr_t>(C) % 16 == 0 && ib % 16 == 0;
+  for (int n = 0; vc && n < p.Ns; ++n) vc = p.nC[n] == n;
+  for (int s = 0; vc && s < p.nseg; ++s) vc = p.seg_sC[s] % 4 == 0;
+  return vc;
+}
+
+template <typename T, typename I>
 static bool launch_gate_t(const GateParams &p, const T *A, const T *B, T *C, dim3 blocks,
                           int threads, int64_t ib, cudaStream_t st) {
-#define TN_GATE_CASE(KS_, NS_)                                                                 \
-  if (p.Ks == KS_ && p.Ns == NS_) {                                                            \
-    k_gate_t<T, KS_, NS_><<<blocks, threads, 0, st>>>(p, A, B, C, ib);                         \
+  const bool vc = gate_vec4(p, C, ib);
+#define TN_GATE_CASE(KS_, NS_, VC_)                                                            \
+  if (p.Ks == KS_ && p.Ns == NS_ && (!VC_ || vc)) {                                            \
+    k_gate_t<T, KS_, NS_, I, VC_><<<blocks, threads, 0, st>>>(p, A, B, C, ib);                 \
     return true;                                                                               \
   }
-  TN_GATE_CASE(1, 1)
-  TN_GATE_CASE(1, 2)
-  TN_GATE_CASE(2, 1)
-  TN_GATE_CASE(2, 2)
-  TN_GATE_CASE(4, 1)
-  TN_GATE_CASE(1, 4)
+  TN_GATE_CASE(1, 1, false)
+  TN_GATE_CASE(1, 2, false)
+  TN_GATE_CASE(2, 1, false)
+  TN_GATE_CASE(2, 2, false)
+  TN_GATE_CASE(4, 1, false)
+  TN_GATE_CASE(1, 4, true)
+  TN_GATE_CASE(1, 4, false)
+  TN_GATE_CASE(2, 16, true)
+  TN_GATE_CASE(2, 16, false)
 #undef TN_GATE_CASE
   return false;
 }
@@ -682,11 +681,13 @@ cudaError_t launch_gate(Dtype dt, const GateParams &p, const void *xA, const voi
                                                       (int32_t *)xC, bt, st);
     if (streamed) return cudaGetLastError();
     dim3 b2(grid_for((p.outer + 1) / 2, threads), bt.B);
-    const bool done = dt == DT_F32
-                          ? launch_gate_t<float>(p, (const float *)xA, (const float *)xB,
-                                                 (float *)xC, b2, threads, bt.ib, st)
-                          : launch_gate_t<int32_t>(p, (const int32_t *)xA, (const int32_t *)xB,
-                                                   (int32_t *)xC, b2, threads, bt.ib, st);
+#define TN_GT(T_)                                                                              \
+  (gate_fits32(p) ? launch_gate_t<T_, int32_t>(p, (const T_ *)xA, (const T_ *)xB, (T_ *)xC, b2, \
+                                               threads, bt.ib, st)                             \
+                  : launch_gate_t<T_, int64_t>(p, (const T_ *)xA, (const T_ *)xB, (T_ *)xC, b2, \
+                                               threads, bt.ib, st))
+    const bool done = dt == DT_F32 ? TN_GT(float) : TN_GT(int32_t);
+#undef TN_GT
     if (done) return cudaGetLastError();
   } else {
     const bool streamed =
@@ -701,33 +702,28 @@ cudaError_t launch_gate(Dtype dt, const GateParams &p, const void *xA, const voi
         return cudaGetLastError();
     }
   }
+#define TN_GATE(T_, COUNT_, R_)                                                                \
+  do {                                                                                         \
+    if (gate_fits32(p))                                                                        \
+      k_gate<T_, COUNT_, R_, int32_t><<<blocks, threads, 0, st>>>(                             \
+          p, (const T_ *)xA, (const T_ *)xB, (T_ *)xC, (const R_ *)nA, (const R_ *)nB,         \
+          (R_ *)nC, ps, bt.ib);                                                                \
+    else                                                                                       \
+      k_gate<T_, COUNT_, R_, int64_t><<<blocks, threads, 0, st>>>(                             \
+          p, (const T_ *)xA, (const T_ *)xB, (T_ *)xC, (const R_ *)nA, (const R_ *)nB,         \
+          (R_ *)nC, ps, bt.ib);                                                                \
+  } while (0)
   if (cnt && ps.r32) {
-    const uint32_t *a = (const uint32_t *)nA, *b = (const uint32_t *)nB;
-    uint32_t *c = (uint32_t *)nC;
-    if (dt == DT_F32)
-      k_gate<float, true, uint32_t><<<blocks, threads, 0, st>>>(
-          p, (const float *)xA, (const float *)xB, (float *)xC, a, b, c, ps, bt.ib);
-    else
-      k_gate<int32_t, true, uint32_t><<<blocks, threads, 0, st>>>(
-          p, (const int32_t *)xA, (const int32_t *)xB, (int32_t *)xC, a, b, c, ps, bt.ib);
-    return cudaGetLastError();
-  }
-  if (dt == DT_F32) {
-    if (cnt)
-      k_gate<float, true><<<blocks, threads, 0, st>>>(p, (const float *)xA, (const float *)xB,
-                                                      (float *)xC, nA, nB, nC, ps, bt.ib);
-    else
-      k_gate<float, false><<<blocks, threads, 0, st>>>(p, (const float *)xA, (const float *)xB,
-                                                       (float *)xC, nA, nB, nC, ps, bt.ib);
+    if (dt == DT_F32) TN_GATE(float, true, uint32_t);
+    else TN_GATE(int32_t, true, uint32_t);
+  } else if (cnt) {
+    if (dt == DT_F32) TN_GATE(float, true, uint64_t);
+    else TN_GATE(int32_t, true, uint64_t);
   } else {
-    if (cnt)
-      k_gate<int32_t, true><<<blocks, threads, 0, st>>>(p, (const int32_t *)xA, (const int32_t *)xB,
-                                                        (int32_t *)xC, nA, nB, nC, ps, bt.ib);
-    else
-      k_gate<int32_t, false><<<blocks, threads, 0, st>>>(p, (const int32_t *)xA,
-                                                         (const int32_t *)xB, (int32_t *)xC, nA, nB,
-                                                         nC, ps, bt.ib);
+    if (dt == DT_F32) TN_GATE(float, false, uint64_t);
+    else TN_GATE(int32_t, false, uint64_t);
   }
+#undef TN_GATE
   return cudaGetLastError();
 }
 

@@ -25,6 +25,8 @@ constexpr int kThreads = 256;   // 3^5 of them own 27 elements each of a 3^8 til
 constexpr int kBlocksPerSm = 4; // 2 x 26 KB of tiles each
 constexpr int kMaxT = 8;
 constexpr int kRun = 81;        // elements of a run: the four fastest legs
+// copies: 3 runs at a time, so a thread keeps its place in the run
+constexpr int kCopyRuns = kThreads / kRun, kCopyThreads = kCopyRuns * kRun;
 constexpr int kB = 27;          // values of a gate's operand at most
 
 struct Gate3 {
@@ -47,6 +49,15 @@ struct Plan3 {
 
 __host__ __device__ constexpr int pow3(int e) { return e == 0 ? 1 : 3 * pow3(e - 1); }
 
+__device__ __forceinline__ float max3(float a, float b, float c) {
+  float r;
+  asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+  return r;
+}
+__device__ __forceinline__ int32_t max3(int32_t a, int32_t b, int32_t c) {
+  return max(max(a, b), c);
+}
+
 // Replace leg J: v'[n] = max_u v[u] + B[u, n], for each digit of register leg K (-1: none).
 template <int J, int K, typename T>
 __device__ __forceinline__ void rep3(T (&v)[27], const T *B, const Gate3 &g) {
@@ -65,7 +76,7 @@ __device__ __forceinline__ void rep3(T (&v)[27], const T *B, const Gate3 &g) {
       const T a = v[e], b = v[e + sj], c = v[e + 2 * sj];
 #pragma unroll
       for (int n = 0; n < 3; ++n)
-        v[e + n * sj] = max(max(a + m[0][n], b + m[1][n]), c + m[2][n]);
+        v[e + n * sj] = max3(a + m[0][n], b + m[1][n], c + m[2][n]);
     }
   }
 }
@@ -119,6 +130,7 @@ __global__ void __launch_bounds__(kThreads, kBlocksPerSm)
   for (int i = threadIdx.x; i < p.ngates; i += kThreads) sG[i] = pl.gate[i];
   for (int i = threadIdx.x; i < p.nhi; i += kThreads) sHi[i] = p.hi_off[i];
   __syncthreads();
+  const int run0 = threadIdx.x / kRun, col = threadIdx.x % kRun;
   auto base_of = [&](int64_t o) {
     int64_t b = 0;
     for (int sg = p.nseg - 1; sg >= 0; --sg) {
@@ -131,10 +143,10 @@ __global__ void __launch_bounds__(kThreads, kBlocksPerSm)
   auto fetch = [&](int64_t o, T *dst) {
     if (o < p.outer) {
       const T *src = A + base_of(o);
-      for (int i = threadIdx.x; i < p.tile; i += kThreads) {
-        const int h = i / kRun;
-        cp_async4(dst + i, src + sHi[h] + (i - h * kRun));
-      }
+      if (threadIdx.x < kCopyThreads)
+#pragma unroll 9
+        for (int h = run0; h < p.nhi; h += kCopyRuns)
+          cp_async4(dst + h * kRun + col, src + sHi[h] + col);
     }
     cp_async_commit();
   };
@@ -178,10 +190,9 @@ __global__ void __launch_bounds__(kThreads, kBlocksPerSm)
       __syncthreads();
     }
     T *dst = C + base_of(o);
-    for (int i = threadIdx.x; i < p.tile; i += kThreads) {
-      const int h = i / kRun;
-      dst[sHi[h] + (i - h * kRun)] = s[i];
-    }
+    if (threadIdx.x < kCopyThreads)
+#pragma unroll 9
+      for (int h = run0; h < p.nhi; h += kCopyRuns) dst[sHi[h] + col] = s[h * kRun + col];
     __syncthreads();   // the next fetch but one overwrites this tile
   }
 }

@@ -1841,18 +1841,19 @@ __device__ __forceinline__ void apply_gate_count(const ChainGate &g, T *s, R *sn
   }
 }
 
-// Copy every gate's B (values, and planes when P > 0) into shared memory.
+// Copy every gate's B (values, and planes when P > 0) into shared memory: all elements of
+// all gates at once (one gate after the other is a chain of load latencies).
 template <typename T, typename R>
 __device__ __forceinline__ void load_gate_operands(const ChainParams &p, const T *X,
                                                    const R *Xn, T *sB, R *sBn,
                                                    int stride_el) {
-  for (int gi = 0; gi < p.ngates; ++gi) {
+  for (int i = threadIdx.x; i < p.ngates * stride_el; i += blockDim.x) {
+    const int gi = i / stride_el, e = i - gi * stride_el;
     const ChainGate &g = p.g[gi];
-    for (int e = threadIdx.x; e < g.nBel; e += blockDim.x) {
-      sB[gi * stride_el + e] = X[g.offB + e];
-      for (int pl = 0; pl < p.P; ++pl)
-        sBn[((int64_t)gi * p.P + pl) * stride_el + e] = Xn[g.offBn + pl * g.planeB + e];
-    }
+    if (e >= g.nBel) continue;
+    sB[i] = X[g.offB + e];
+    for (int pl = 0; pl < p.P; ++pl)
+      sBn[((int64_t)gi * p.P + pl) * stride_el + e] = Xn[g.offBn + pl * g.planeB + e];
   }
 }
 

@@ -14,7 +14,7 @@ CSRC = os.path.join(HERE, "csrc")
 OUT_DIR = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libtn.so")
 SOURCES = ["kernels.cu", "gate_count_i32.cu", "gate_count_f32.cu", "chain_sat.cu", "small_run.cu", "trace_walk.cu",
-           "sample_frontier.cu", "chain3.cu",
+           "sample_frontier.cu", "chain3.cu", "gate_sum.cu",
            "noalloc.cu", "planner.cpp",
            "program.cpp", "api.cpp", "jit.cpp", "sampler.cpp"]
 # headers the run-time compiled chain kernels include (embedded into jit.cpp)

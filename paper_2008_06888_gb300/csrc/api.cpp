@@ -106,6 +106,7 @@ const char *op_name(OpKind k) {
     case OP_TRACE: return "traceback";
     case OP_CHAIN: return "gate_chain";
     case OP_SMALL: return "small_steps";
+    case OP_GSUM: return "gate_product";
   }
   return "op";
 }
@@ -294,6 +295,7 @@ int op_kind_slot(OpKind k) {
     case OP_PERM: return 1;
     case OP_GATE: return 2;
     case OP_SMALL: return 2;
+    case OP_GSUM: return 2;
     case OP_GEMM: return 3;
     case OP_TRACE: return 4;
     case OP_CHAIN: return 6;
@@ -390,6 +392,19 @@ tn_status run_ops(tn_ctx *ctx, Program &p, int op_begin, int op_end, cudaStream_
           e = launch_chain(p.dt, p.chains[op.idx], ar, X(op.in0), Nn(op.in0), X(op.out),
                            Nn(op.out), ps, bt, st);
         break;
+      case OP_GSUM: {
+        const SumOp &so = p.gsums[op.idx];
+        const void *A[TN_SUM_MAX_G], *B[TN_SUM_MAX_G];
+        const uint64_t *nA[TN_SUM_MAX_G];
+        for (int g = 0; g < so.p.n; ++g) {
+          A[g] = X(so.A[g]);
+          B[g] = X(so.B[g]);
+          nA[g] = p.P > 0 ? Nn(so.A[g]) : nullptr;
+        }
+        e = launch_gate_sum(p.dt, p.P > 0, so.p, A, B, nA, X(op.out),
+                            p.P > 0 ? Nn(op.out) : nullptr, bt, st);
+        break;
+      }
       case OP_SMALL: {
         const SmallRun &r = p.smalls[op.idx];
         e = launch_small(p.dt, p.sat, p.d_small + r.desc_off, r.desc_len, ar, bt, st);
@@ -1682,6 +1697,7 @@ tn_status tn_energy_noalloc(tn_ctx *ctx, const float *J_dev, const float *h_dev,
         break;
       case OP_TRACE:
       case OP_SMALL:
+      case OP_GSUM:
         break;
       case OP_CHAIN:
         e = launch_chain(p.dt, p.chains[op.idx], base, X(op.in0), nullptr, X(op.out), nullptr, ps,

@@ -130,6 +130,23 @@ cudaError_t launch_schain(const ChainParams &p, const char *arena, const void *A
                           const uint64_t *An, void *Cx, uint64_t *Cn, const Batch &bt,
                           cudaStream_t st);
 
+// Sum of n = 2 or 4 gate contractions over the same output indices (gate_sum.cu):
+// n = 2: G0 + G1, n = 4: (G0 + G1) + (G2 + G3); counts multiply.  gate_sum_leaf: whether
+// a gate has the form it takes; gate_sum_add: append one (false: its outputs differ).
+constexpr int TN_SUM_MAX_G = 4;
+struct GateSum {
+  int32_t n = 0, nseg = 0, Ns = 0;
+  int64_t outer = 0;
+  int32_t seg_size[TN_MAX_SEG], seg_sh[TN_MAX_SEG], seg_sC[TN_MAX_SEG];
+  int32_t seg_sA[TN_SUM_MAX_G][TN_MAX_SEG];
+  int32_t kA[TN_SUM_MAX_G][2], kB[TN_SUM_MAX_G][2], nB[TN_SUM_MAX_G][TN_GATE_MAX_N];
+};
+bool gate_sum_leaf(const GateParams &g, bool cnt);
+bool gate_sum_add(GateSum *p, const GateParams &g);
+cudaError_t launch_gate_sum(Dtype dt, bool cnt, const GateSum &p, const void *const *A,
+                            const void *const *B, const uint64_t *const *nA, void *C,
+                            uint64_t *nC, const Batch &bt, cudaStream_t st);
+
 // Fused gate chain of q = 3 values (chain3.cu).
 cudaError_t launch_chain3(Dtype dt, const ChainParams &p, const char *arena, const void *A,
                           void *C, const Batch &bt, cudaStream_t st);

@@ -1198,6 +1198,118 @@ struct Builder {
     return true;
   }
 
+  // ---- products of gate contractions (SumOp)
+  //
+  // A Hadamard step (one product per element, operands and output in one layout) whose
+  // operands are gate contractions, or products of two of them, that nothing else reads
+  // becomes one step with them.  Forward-only programs: a traceback reads intermediates.
+  // From 2^14 elements on; below, a launch less is what the small runs give already.
+  static constexpr int64_t kSumMin = 1 << 14;
+  void fuse_sums() {
+    const int n = (int)pr.ops.size();
+    std::vector<int> prod(pr.bufs.size(), -1), nuse(pr.bufs.size(), 0);
+    for (int i = 0; i < n; ++i)
+      if (pr.ops[i].out.buf >= 0) prod[pr.ops[i].out.buf] = i;
+    for (auto &u : uses) nuse[u.second]++;
+    std::vector<int> into(n, -1);   // the step an op became part of
+    for (int i = 0; i < n; ++i) {
+      Op &op = pr.ops[i];
+      if (op.kind != OP_GATE) continue;
+      const GateParams &h = pr.gates[op.idx];
+      if (!h.hasB || h.Ks != 1 || h.Ns != 1 || h.nseg != 1 || h.outer < kSumMin ||
+          h.seg_sA[0] != 1 || h.seg_sB[0] != 1 || h.seg_sC[0] != 1)
+        continue;
+      const Loc in[2] = {op.in0, op.in1};
+      SumOp so;
+      int from[2];
+      bool ok = true;
+      for (int j = 0; j < 2 && ok; ++j) {
+        // written by one step, read by this one (and by nothing else)
+        from[j] = in[j].buf >= 0 && nuse[in[j].buf] == 2 ? prod[in[j].buf] : -1;
+        ok = from[j] >= 0 && in[j].xoff == 0 && in[j].plane == h.outer;
+        if (!ok) break;
+        const Op &f = pr.ops[from[j]];
+        if (f.kind == OP_GATE && gate_sum_leaf(pr.gates[f.idx], P > 0) &&
+            pr.gates[f.idx].outer * pr.gates[f.idx].Ns == h.outer) {
+          ok = gate_sum_add(&so.p, pr.gates[f.idx]);
+          so.A.push_back(f.in0);
+          so.B.push_back(f.in1);
+        } else {
+          ok = false;
+        }
+      }
+      if (!ok && from[0] >= 0 && in[1].buf >= 0 && nuse[in[1].buf] == 2 && prod[in[1].buf] >= 0 &&
+          in[0].plane == h.outer && in[1].plane == h.outer) {
+        // two products of two
+        const Op &f0 = pr.ops[from[0]], &f1 = pr.ops[prod[in[1].buf]];
+        if (f0.kind == OP_GSUM && f1.kind == OP_GSUM && pr.gsums[f0.idx].p.n == 2 &&
+            pr.gsums[f1.idx].p.n == 2) {
+          so = pr.gsums[f0.idx];
+          const SumOp &t = pr.gsums[f1.idx];
+          ok = so.p.nseg == t.p.nseg && so.p.Ns == t.p.Ns && so.p.outer == t.p.outer;
+          for (int s = 0; ok && s < t.p.nseg; ++s)
+            ok = so.p.seg_size[s] == t.p.seg_size[s] && so.p.seg_sC[s] == t.p.seg_sC[s];
+          if (ok) {
+            for (int g = 0; g < 2; ++g) {
+              std::copy(t.p.seg_sA[g], t.p.seg_sA[g] + TN_MAX_SEG, so.p.seg_sA[2 + g]);
+              std::copy(t.p.kA[g], t.p.kA[g] + 2, so.p.kA[2 + g]);
+              std::copy(t.p.kB[g], t.p.kB[g] + 2, so.p.kB[2 + g]);
+              std::copy(t.p.nB[g], t.p.nB[g] + TN_GATE_MAX_N, so.p.nB[2 + g]);
+              so.A.push_back(t.A[g]);
+              so.B.push_back(t.B[g]);
+            }
+            so.p.n = 4;
+            from[1] = prod[in[1].buf];
+          }
+        }
+      }
+      if (!ok || (so.p.n != 2 && so.p.n != 4)) continue;
+      for (int j = 0; j < 2; ++j) {
+        into[from[j]] = i;
+        op.macs += pr.ops[from[j]].macs;
+      }
+      op.kind = OP_GSUM;
+      op.idx = (int)pr.gsums.size();
+      op.in0 = op.in1 = Loc{};
+      op.bytes = (double)h.outer * elem_bytes();
+      for (size_t g = 0; g < so.A.size(); ++g)
+        op.bytes += (double)(so.A[g].plane + so.B[g].plane) * elem_bytes();
+      pr.gsums.push_back(so);
+    }
+    // drop the absorbed steps; their operands are used by the step they went into
+    std::vector<int> at(n + 1, 0);
+    std::vector<Op> ops;
+    for (int i = 0; i < n; ++i) {
+      at[i] = (int)ops.size();
+      if (into[i] < 0) ops.push_back(pr.ops[i]);
+    }
+    at[n] = (int)ops.size();
+    if ((int)ops.size() == n) return;
+    std::vector<std::pair<int, int>> nu;
+    for (auto &u : uses) {
+      int i = u.first;
+      const bool dead_out = i < n && into[i] >= 0 && pr.ops[i].out.buf == u.second;
+      while (i < n && into[i] >= 0) i = into[i];
+      // the absorbed steps' outputs are gone: no longer written, no longer read
+      const int w = prod[u.second];
+      if (dead_out || (w >= 0 && into[w] >= 0)) continue;
+      nu.push_back({at[i], u.second});
+    }
+    uses.swap(nu);
+    pr.fwd_end = at[pr.fwd_end];
+    pr.ops.swap(ops);
+    for (size_t b = 0; b < pr.bufs.size(); ++b) {
+      pr.bufs[b].first = 1 << 30;
+      pr.bufs[b].last = -1;
+      if (prod[b] >= 0 && into[prod[b]] >= 0) pr.bufs[b].bytes = kAlign;
+    }
+    for (auto &u : uses) {
+      BufInfo &b = pr.bufs[u.second];
+      b.first = std::min(b.first, u.first);
+      b.last = std::max(b.last, u.first);
+    }
+  }
+
   // ---- runs of small steps (SmallRun)
   //
   // A step counts as small up to kSmallWork products: at that size one block takes
@@ -1354,6 +1466,9 @@ struct Builder {
       flush_trace();
     }
     use(pr.root, (int)pr.ops.size());
+    if (small_runs && mode != PM_CONFIG && (P == 0 || pr.sat) &&
+        std::getenv("TN_NO_GATE_SUM") == nullptr)
+      fuse_sums();
     if (small_runs && (P == 0 || pr.sat) && std::getenv("TN_NO_SMALL_RUNS") == nullptr)
       schedule_small();
     return true;

@@ -24,7 +24,7 @@ struct BufInfo {
   int64_t off = -1;
 };
 
-enum OpKind { OP_LEAVES, OP_PERM, OP_GATE, OP_GEMM, OP_TRACE, OP_CHAIN, OP_SMALL };
+enum OpKind { OP_LEAVES, OP_PERM, OP_GATE, OP_GEMM, OP_TRACE, OP_CHAIN, OP_SMALL, OP_GSUM };
 
 struct Op {
   OpKind kind;
@@ -43,6 +43,12 @@ struct SmallRun {
   std::vector<int> level;
   int64_t desc_off = 0;
   int desc_len = 0;
+};
+
+// A product of gate contractions (gate_sum.cu) and its operands.
+struct SumOp {
+  GateSum p;
+  std::vector<Loc> A, B;
 };
 
 // One traceback launch of a q = 2 plan with folded chains: records [begin, begin + n)
@@ -71,6 +77,7 @@ struct Program {
   std::vector<GemmParams> gemms;
   std::vector<PermParams> perms;
   std::vector<SmallRun> smalls;
+  std::vector<SumOp> gsums;
   std::vector<int32_t> small_desc;                  // descriptors of every run
   std::vector<ChainParams> chains;                  // fused gate chains
   std::vector<const void *> chain_jit;              // their compiled kernels (nullptr: interpreted)

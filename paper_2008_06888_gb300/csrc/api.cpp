@@ -407,7 +407,8 @@ tn_status run_ops(tn_ctx *ctx, Program &p, int op_begin, int op_end, cudaStream_
       }
       case OP_SMALL: {
         const SmallRun &r = p.smalls[op.idx];
-        e = launch_small(p.dt, p.sat, p.d_small + r.desc_off, r.desc_len, ar, bt, st);
+        e = launch_small(p.dt, p.sat, p.d_small + r.desc_off, r.desc_len, r.scratch, ar, bt,
+                         st);
         break;
       }
     }

@@ -108,15 +108,18 @@ cudaError_t launch_frontier_sample(const FrontierPlan &p, const FrontierStep *st
                                    cudaStream_t st);
 
 // A run of small steps in one launch, one block per instance.  Descriptors (32-bit
-// words): {steps, levels}, level starts [levels + 1], per step its first output within
-// its level, per step the word of its body, then the bodies: 64-bit offsets of the
-// values of A, B (-1: none) and C in elements and of their counts in 8-byte words,
-// digits, K, N, unit B counts, outputs, then (size, stride in A, stride in B) of each
-// outer digit (slowest first), (offset in A, in B) of each k, the offset in B of each n.
-// sat: one plane of saturating 64-bit counts.
+// words): {steps, levels}, level starts [levels + 1], outputs of each level, per step its
+// first output within its level, per step the word of its body, then the bodies: 64-bit
+// offsets of the values of A, B (-1: none) and C (-1: not stored) in elements and of their
+// counts in 8-byte words, digits, K, N, unit B counts, shared-memory elements of A, B and C
+// (-1: not there), then (size, stride in A, stride in B) of each outer digit (slowest
+// first), (offset in A, in B) of each k, the offset in B of each n (N > 1).  words is a
+// multiple of 4; scratch: shared-memory elements.  sat: one plane of saturating 64-bit
+// counts.
 constexpr int kSmallMaxWords = 40 * 1024;     // descriptor words of a run at most
-cudaError_t launch_small(Dtype dt, bool sat, const int32_t *d_desc, int words, char *arena,
-                         const Batch &bt, cudaStream_t st);
+constexpr int kSmallScratch = 5 * 1024;       // shared-memory elements at most (12 bytes each)
+cudaError_t launch_small(Dtype dt, bool sat, const int32_t *d_desc, int words, int scratch,
+                         char *arena, const Batch &bt, cudaStream_t st);
 
 // Fused gate chain over tiles of the big tensor (values; planes when P > 0).
 cudaError_t launch_chain(Dtype dt, const ChainParams &p, const char *arena, const void *Ax,

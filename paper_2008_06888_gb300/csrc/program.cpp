@@ -1330,7 +1330,7 @@ struct Builder {
   int small_words(const Op &op) const {   // an upper bound of its descriptor
     const int seg = op.kind == OP_GATE ? pr.gates[op.idx].nseg : op.kind == OP_PERM ? 14 : 3;
     const int ks = op.kind == OP_GATE ? pr.gates[op.idx].Ks : op.kind == OP_GEMM ? 64 : 1;
-    return 24 + 3 * seg + 2 * ks + TN_GATE_MAX_N;
+    return 32 + 3 * seg + 2 * ks + TN_GATE_MAX_N;
   }
 
   // Every small step of the forward pass moves up to right behind the last launch it
@@ -1370,7 +1370,7 @@ struct Builder {
       std::stable_sort(run.begin(), run.end(), [&](int x, int y) { return level[x] < level[y]; });
       for (size_t k = 0; k < run.size();) {
         SmallRun sr;
-        int words = 8;
+        int words = 64;
         size_t e = k;
         for (; e < run.size(); ++e) {
           const int w = small_words(pr.ops[run[e]]) + 3;
@@ -1512,6 +1512,7 @@ struct SmallBody {
   int64_t offA = 0, offB = -1, offC = 0;   // element offsets of the values (B: -1 none)
   int64_t nA = 0, nB = 0, nC = 0;          // and of the counts, in 8-byte words
   int nout = 0, unitB = 1;
+  int sA = -1, sB = -1, sC = -1;           // shared-memory elements (-1: not there)
   int Ks = 1, Ns = 1;
   std::vector<int64_t> seg_size, seg_sA, seg_sB;   // outer digits, slowest first
   std::vector<int64_t> kA, kB, nBo;        // offsets of k in A and B, of n in B
@@ -1523,7 +1524,7 @@ static std::vector<int32_t> encode_small(const std::vector<SmallBody> &ops,
   const int n = (int)ops.size(), nlev = (int)level.size() - 1;
   std::vector<int32_t> w{n, nlev};
   w.insert(w.end(), level.begin(), level.end());
-  const size_t first = w.size(), body = first + n;
+  const size_t tot = w.size(), first = tot + nlev, body = first + n;
   w.resize(body + n);
   auto put64 = [&](int64_t v) {
     w.push_back((int32_t)(uint32_t)(uint64_t)v);
@@ -1541,7 +1542,7 @@ static std::vector<int32_t> encode_small(const std::vector<SmallBody> &ops,
       w.push_back(o.Ks);
       w.push_back(o.Ns);
       w.push_back(o.unitB);
-      w.push_back(o.nout);
+      for (int v : {o.sA, o.sB, o.sC}) w.push_back(v);
       for (size_t s = 0; s < o.seg_size.size(); ++s) {
         w.push_back((int32_t)o.seg_size[s]);
         w.push_back((int32_t)o.seg_sA[s]);
@@ -1554,8 +1555,83 @@ static std::vector<int32_t> encode_small(const std::vector<SmallBody> &ops,
       if (o.Ns > 1)
         for (int k = 0; k < o.Ns; ++k) w.push_back((int32_t)o.nBo[k]);
     }
+    w[tot + l] = at;
   }
+  while (w.size() % 4) w.push_back(0);   // runs start on 16-byte boundaries
   return w;
+}
+
+// Shared-memory places for a run: the leaves (copied by a step in front, when they fit half
+// of it) and every output that later levels of the run read, first fit, an output's place
+// free again behind the last level that reads it.  Returns the elements taken.
+static int place_small(const Program &pr, const SmallRun &r, std::vector<SmallBody> *ops,
+                       std::vector<int> *level) {
+  const int nlev = (int)r.level.size() - 1;
+  struct Place { int off, size, from, to; };   // levels [from, to]
+  std::vector<Place> taken;
+  int peak = 0;
+  auto place = [&](int size, int from, int to, int cap) {
+    std::vector<std::pair<int, int>> busy;
+    for (const Place &p : taken)
+      if (p.from <= to && from <= p.to) busy.push_back({p.off, p.off + p.size});
+    std::sort(busy.begin(), busy.end());
+    int off = 0;
+    for (auto &b : busy) {
+      if (b.first >= off + size) break;
+      off = std::max(off, b.second);
+    }
+    if (off + size > cap) return -1;
+    taken.push_back({off, size, from, to});
+    peak = std::max(peak, off + size);
+    return off;
+  };
+  const int64_t nleaf = pr.leaves_loc.plane;
+  bool reads_leaves = false;
+  std::map<int, std::pair<int, int>> made;   // buffer -> (level written, last level read)
+  for (int l = 0; l < nlev; ++l)
+    for (int i = r.level[l]; i < r.level[l + 1]; ++i) {
+      for (const Loc *x : {&r.ops[i].in0, &r.ops[i].in1}) {
+        reads_leaves = reads_leaves || x->buf == pr.leaves_loc.buf;
+        if (made.count(x->buf)) made[x->buf].second = l;
+      }
+      made[r.ops[i].out.buf] = {l, -1};
+    }
+  std::map<int, int> at;   // buffer -> shared-memory element
+  if (reads_leaves && nleaf <= kSmallScratch / 2) {
+    const int off = place((int)nleaf, 0, nlev, kSmallScratch);
+    at[pr.leaves_loc.buf] = off;
+  }
+  for (int l = 0; l < nlev; ++l)
+    for (int i = r.level[l]; i < r.level[l + 1]; ++i) {
+      SmallBody &b = (*ops)[i];
+      auto find = [&](const Loc &x) {
+        auto it = at.find(x.buf);
+        return it == at.end() ? -1 : it->second + (int)(x.xoff / 4);
+      };
+      b.sA = find(r.ops[i].in0);
+      b.sB = b.offB >= 0 ? find(r.ops[i].in1) : -1;
+      const int last = made[r.ops[i].out.buf].second;
+      if (last < 0) continue;
+      b.sC = place(b.nout, l, last, kSmallScratch);
+      if (b.sC >= 0) at[r.ops[i].out.buf] = b.sC;
+    }
+  *level = r.level;
+  if (at.count(pr.leaves_loc.buf)) {
+    SmallBody c;   // the copy of the leaves: its output stays in shared memory
+    c.offA = abs_off(pr, pr.leaves_loc) / 4;
+    c.nA = (pr.bufs[pr.leaves_loc.buf].off + pr.leaves_loc.noff) / 8;
+    c.offC = -1;
+    c.sC = at[pr.leaves_loc.buf];
+    c.nout = (int)nleaf;
+    c.seg_size = {nleaf};
+    c.seg_sA = {1};
+    c.seg_sB = {0};
+    c.kA = c.kB = c.nBo = {0};
+    ops->insert(ops->begin(), c);
+    for (int &x : *level) ++x;
+    level->insert(level->begin(), 0);
+  }
+  return peak;
 }
 
 // One traceback record as k_walk reads it.  Plain: {0, legs of A, legs of B, contracted
@@ -1755,7 +1831,9 @@ bool build_program(const Net &net, const Plan &plan, ProgMode mode, Dtype dt, in
   for (SmallRun &r : pr->smalls) {
     std::vector<SmallBody> bodies;
     for (const Op &op : r.ops) bodies.push_back(small_body(*pr, op));
-    const std::vector<int32_t> w = encode_small(bodies, r.level);
+    std::vector<int> level;
+    r.scratch = place_small(*pr, r, &bodies, &level);
+    const std::vector<int32_t> w = encode_small(bodies, level);
     r.desc_off = (int64_t)pr->small_desc.size();
     r.desc_len = (int)w.size();
     pr->small_desc.insert(pr->small_desc.end(), w.begin(), w.end());

@@ -42,7 +42,7 @@ struct SmallRun {
   std::vector<Op> ops;
   std::vector<int> level;
   int64_t desc_off = 0;
-  int desc_len = 0;
+  int desc_len = 0, scratch = 0;       // descriptor words, shared-memory elements
 };
 
 // A product of gate contractions (gate_sum.cu) and its operands.

@@ -1995,6 +1995,9 @@ __device__ void trace_chain(const ChainTrace &ct, const T *X, int8_t *state, int
   const ChainParams &p = ct.p;
   __shared__ int sx, snrep, srl[TN_CHAIN_MAX_T];        // final local index; replaced legs
   __shared__ int sss[TN_CHAIN_MAX_G], sbs[TN_CHAIN_MAX_G][2], sfix[TN_CHAIN_MAX_G];
+  // ceil(2^32 / stride): quotients of sub-tile indices (below 2^12, strides below 2^11)
+  // are one high product
+  __shared__ unsigned smg[TN_CHAIN_MAX_G], smb[TN_CHAIN_MAX_G][2];
   auto digit = [](int x, int s) { return (x / s) % Q; };
   if (threadIdx.x < 32) {
     const int lane = threadIdx.x;
@@ -2049,10 +2052,13 @@ __device__ void trace_chain(const ChainTrace &ct, const T *X, int8_t *state, int
     for (int j = 0; j < 2; ++j) {
       const int r = j < g.nb ? substride(g.lsb[j]) : 0;
       sbs[threadIdx.x][j] = r;
+      smb[threadIdx.x][j] = r > 1 ? 0xffffffffu / r + 1 : 0;
       if (j < g.nb && r == 0) fix += digit(x, g.lsb[j]) * (int)g.sBb[j];
     }
     sfix[threadIdx.x] = fix;
-    sss[threadIdx.x] = g.kind == 0 ? substride(g.ls) : 0;
+    const int ss = g.kind == 0 ? substride(g.ls) : 0;
+    sss[threadIdx.x] = ss;
+    smg[threadIdx.x] = ss > 1 ? 0xffffffffu / ss + 1 : 0;
   }
   load_gate_operands<T, uint64_t>(p, X, nullptr, sB, nullptr, kGateBMax);
   const int64_t base = *sbase;
@@ -2065,38 +2071,46 @@ __device__ void trace_chain(const ChainTrace &ct, const T *X, int8_t *state, int
     buf[y] = X[base + tile_elem_off<Q>(p, xl)];
   }
   __syncthreads();
+  auto quick = [](int y, unsigned magic) {   // digit of sub-tile index y (magic 0: stride 1)
+    return (int)((magic ? __umulhi((unsigned)y, magic) : (unsigned)y) % Q);
+  };
   auto boff = [&](int gi, int y) {   // operand offset of sub-tile element y
     int o = sfix[gi];
     for (int j = 0; j < 2; ++j)
-      if (sbs[gi][j] > 0) o += digit(y, sbs[gi][j]) * (int)p.g[gi].sBb[j];
+      if (sbs[gi][j] > 0) o += quick(y, smb[gi][j]) * (int)p.g[gi].sBb[j];
     return o;
   };
+  // Diagonal gates act on an element by itself, in place: the state kept in front of a
+  // replace gate includes those that precede it, and only replace gates are barriers.
+  T *cur = buf;
   for (int gi = 0; gi < p.ngates; ++gi) {
     const ChainGate &g = p.g[gi];
-    const T *src = buf + (int64_t)gi * sub, *B = sB + gi * kGateBMax;
-    T *dst = buf + (int64_t)(gi + 1) * sub;
-    const int ss = sss[gi];
+    const T *B = sB + gi * kGateBMax;
     if (g.kind == 0) {
+      const int ss = sss[gi];
+      T *dst = cur + sub;
+      __syncthreads();
       for (int y = threadIdx.x; y < sub; y += blockDim.x) {
-        const int v = digit(y, ss), y0 = y - v * ss, bo = boff(gi, y0) + v * (int)g.sBn;
-        T best = src[y0] + B[bo];
+        const int v = quick(y, smg[gi]), y0 = y - v * ss, bo = boff(gi, y0) + v * (int)g.sBn;
+        T best = cur[y0] + B[bo];
 #pragma unroll
-        for (int u = 1; u < Q; ++u) best = max(best, src[y0 + u * ss] + B[bo + u * (int)g.sBk]);
+        for (int u = 1; u < Q; ++u) best = max(best, cur[y0 + u * ss] + B[bo + u * (int)g.sBk]);
         dst[y] = best;
       }
+      cur = dst;
     } else {
-      for (int y = threadIdx.x; y < sub; y += blockDim.x) dst[y] = src[y] + B[boff(gi, y)];
+      for (int y = threadIdx.x; y < sub; y += blockDim.x) cur[y] = cur[y] + B[boff(gi, y)];
     }
-    __syncthreads();
   }
   if (threadIdx.x == 0) {
     int y = yx;
     for (int gi = p.ngates - 1; gi >= 0; --gi) {
       const ChainGate &g = p.g[gi];
       if (g.kind != 0) continue;
-      const T *src = buf + (int64_t)gi * sub;
+      cur -= sub;
+      const T *src = cur;
       const T *gB = sB + gi * kGateBMax;
-      const int ss = sss[gi], v = digit(y, ss), y0 = y - v * ss;
+      const int ss = sss[gi], v = quick(y, smg[gi]), y0 = y - v * ss;
       const int64_t bo = boff(gi, y0);
       int bu = 0;
       T best = src[y0] + gB[bo + v * g.sBn];
@@ -2991,7 +3005,9 @@ cudaError_t launch_rchain(Dtype dt, const ChainParams &p, const char *arena, con
 // Steps are processed in order (the host lists them top-down).  For each, the
 // fixed legs select the slice of A and B, the block finds the first k that
 // maximises A + B, and the contracted spins take the digits of k.
-constexpr int kTraceThreads = 128;  // all threads copy records and build tables; warp 0 walks
+// all threads copy records, build tables and replay chains; warp 0 walks.  q = 3 replays up
+// to 3^7 states per gate and has more threads for it.
+template <int Q> constexpr int kTraceThreads = Q == 3 ? 512 : 128;
 
 // (value, k) pair reduction keeping the larger value, the smaller k on ties.
 template <typename T>
@@ -3008,7 +3024,7 @@ __device__ __forceinline__ void argmax_merge(T &v, int &k, T v2, int k2) {
 // k maximising A + B and assigns the contracted spins.  Chain records:
 // trace_chain above.
 template <typename T, int Q>
-__global__ void __launch_bounds__(kTraceThreads) k_trace(const TraceStep *__restrict__ steps,
+__global__ void __launch_bounds__(kTraceThreads<Q>) k_trace(const TraceStep *__restrict__ steps,
                                                          int nsteps,
                                                          const ChainTrace *__restrict__ chains,
                                                          const char *__restrict__ arena,
@@ -3030,7 +3046,7 @@ __global__ void __launch_bounds__(kTraceThreads) k_trace(const TraceStep *__rest
   // records are copied into shared memory by all threads; the copy of record
   // s + 1 is in flight (registers) while record s is walked
   constexpr int kWords = (int)((sizeof(ChainTrace) + 7) / 8);
-  constexpr int kPer = (kWords + kTraceThreads - 1) / kTraceThreads;
+  constexpr int NT = kTraceThreads<Q>, kPer = (kWords + NT - 1) / NT;
   __shared__ __align__(16) unsigned long long srec2[2][kWords];
   unsigned long long tmp[kPer];
   auto fetch = [&](int s2) {
@@ -3041,14 +3057,14 @@ __global__ void __launch_bounds__(kTraceThreads) k_trace(const TraceStep *__rest
     const int words = (int)((ch >= 0 ? sizeof(ChainTrace) : sizeof(TraceStep)) / 8);
 #pragma unroll
     for (int i = 0; i < kPer; ++i) {
-      const int w = threadIdx.x + i * kTraceThreads;
+      const int w = threadIdx.x + i * NT;
       tmp[i] = w < words ? src[w] : 0ull;
     }
   };
   auto put = [&](unsigned long long *dst) {
 #pragma unroll
     for (int i = 0; i < kPer; ++i) {
-      const int w = threadIdx.x + i * kTraceThreads;
+      const int w = threadIdx.x + i * NT;
       if (w < kWords) dst[w] = tmp[i];
     }
   };
@@ -3155,7 +3171,7 @@ static cudaError_t launch_trace_t(const TraceStep *d_steps, int nsteps, const Ch
     if (e != cudaSuccess) return e;
     configured = smem;
   }
-  k_trace<T, Q><<<bt.B, kTraceThreads, smem, st>>>(d_steps, nsteps, chains, arena, state, nspins,
+  k_trace<T, Q><<<bt.B, kTraceThreads<Q>, smem, st>>>(d_steps, nsteps, chains, arena, state, nspins,
                                                    err, bt.ib);
   return cudaGetLastError();
 }

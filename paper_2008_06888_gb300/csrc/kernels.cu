@@ -755,66 +755,92 @@ __device__ __forceinline__ int32_t tmac2(int32_t acc, int32_t a0, int32_t b0, in
 
 constexpr int GBM = 128, GBN = 128, GBK = 16, GPAD = 4;
 
-template <typename T>
-__device__ __forceinline__ void gemm_load_tile(const GemmParams &p, const T *Ab, const T *Bb,
-                                               int64_t m0, int64_t n0, int64_t k0, T *As, T *Bs) {
+// One operand's k slab of a tile, ROWS rows (or columns) x 16 k, into dst[k][row] by NT
+// threads: consecutive threads along k (kfast) or along the rows, whichever is contiguous
+// in memory; a thread's elements are a constant step apart, and whole slabs need no bounds.
+template <int ROWS, int NT, typename T>
+__device__ __forceinline__ void gemm_load_side(const T *src, int64_t sR, int64_t sK, bool kfast,
+                                               int64_t rows, int64_t kr, T *dst) {
+  constexpr int L = ROWS + GPAD, PER = ROWS * GBK / NT;
   const int tid = threadIdx.x;
-  const T *a0 = Ab + m0 * p.sAm + k0 * p.sAk;
-  const T *b0 = Bb + k0 * p.sBk + n0 * p.sBn;
-  const int64_t mr = p.M - m0, kr = p.K - k0, nr = p.N - n0;
-  // A: GBM x GBK elements into As[k][m]
+  const bool whole = rows >= ROWS && kr >= GBK;
+  if (kfast) {
+    constexpr int DR = NT / GBK;
+    const int r0 = tid / GBK, k = tid % GBK;
+    const T *q = src + r0 * sR + k * sK;
+    T *d = dst + k * L + r0;
+    const int64_t step = DR * sR;
+    if (whole) {
 #pragma unroll 2
-  for (int r = 0; r < (GBM * GBK) / 256; ++r) {
-    const int idx = tid + r * 256;
-    int m, k;
-    if (p.sAk == 1) { m = idx / GBK; k = idx % GBK; } else { k = idx / GBM; m = idx % GBM; }
-    T *dst = As + k * (GBM + GPAD) + m;
-    if (m < mr && k < kr) cp_async4(dst, a0 + m * p.sAm + k * p.sAk);
-    else *dst = Lim<T>::neg();
-  }
-  // B: GBK x GBN elements into Bs[k][n]
+      for (int i = 0; i < PER; ++i, q += step) cp_async4(d + i * DR, q);
+    } else {
 #pragma unroll 2
-  for (int r = 0; r < (GBN * GBK) / 256; ++r) {
-    const int idx = tid + r * 256;
-    int n, k;
-    if (p.sBn == 1) { k = idx / GBN; n = idx % GBN; } else { n = idx / GBK; k = idx % GBK; }
-    T *dst = Bs + k * (GBN + GPAD) + n;
-    if (n < nr && k < kr) cp_async4(dst, b0 + k * p.sBk + n * p.sBn);
-    else *dst = Lim<T>::neg();
+      for (int i = 0; i < PER; ++i, q += step) {
+        if (r0 + i * DR < rows && k < kr) cp_async4(d + i * DR, q);
+        else d[i * DR] = Lim<T>::neg();
+      }
+    }
+  } else {
+    constexpr int DK = NT / ROWS;
+    const int r0 = tid % ROWS, k = tid / ROWS;
+    const T *q = src + r0 * sR + k * sK;
+    T *d = dst + k * L + r0;
+    const int64_t step = DK * sK;
+    if (whole) {
+#pragma unroll 2
+      for (int i = 0; i < PER; ++i, q += step) cp_async4(d + i * DK * L, q);
+    } else {
+#pragma unroll 2
+      for (int i = 0; i < PER; ++i, q += step) {
+        if (r0 < rows && k + i * DK < kr) cp_async4(d + i * DK * L, q);
+        else d[i * DK * L] = Lim<T>::neg();
+      }
+    }
   }
 }
 
-template <typename T>
-__global__ void __launch_bounds__(256, 2) k_mpgemm(const GemmParams p, const T *__restrict__ A,
-                                                   const T *__restrict__ B, T *__restrict__ C,
-                                                   int64_t ib) {
+// General strides and ragged sizes: BM x BN tiles by 8 x 8 outputs per thread.  128 x 128,
+// or 64 x 64 where that wastes less on the edges or leaves fewer SMs idle (the tuner
+// decides; 5 x 777 x 1001 x 333 INT32, A transposed: 138 us with one copy address per
+// element and 128 x 128 tiles alone, 114 now).
+template <typename T, int BM, int BN, int MINB>
+__global__ void __launch_bounds__(BM *BN / 64, MINB)
+    k_mpgemm(const GemmParams p, const T *__restrict__ A, const T *__restrict__ B,
+             T *__restrict__ C, int64_t ib) {
+  constexpr int NT = BM * BN / 64, HM = BM / 2, HN = BN / 2;
   A = inst_ptr(A, ib);
   B = inst_ptr(B, ib);
   C = inst_ptr(C, ib);
-  __shared__ __align__(16) T As[2][GBK][GBM + GPAD];
-  __shared__ __align__(16) T Bs[2][GBK][GBN + GPAD];
-  const int64_t mt = (p.M + GBM - 1) / GBM, nt = (p.N + GBN - 1) / GBN;
+  __shared__ __align__(16) T As[2][GBK][BM + GPAD];
+  __shared__ __align__(16) T Bs[2][GBK][BN + GPAD];
+  const int64_t mt = (p.M + BM - 1) / BM, nt = (p.N + BN - 1) / BN;
   const int64_t tiles = p.batch * mt * nt;
-  const int tid = threadIdx.x, tx = tid % 16, ty = tid / 16;
+  const int tid = threadIdx.x, tx = tid % (BN / 8), ty = tid / (BN / 8);
   const int64_t ksteps = (p.K + GBK - 1) / GBK;
   for (int64_t t = blockIdx.x; t < tiles; t += gridDim.x) {
     const int64_t b = t / (mt * nt);
     const int64_t rem = t % (mt * nt);
-    const int64_t m0 = (rem / nt) * GBM, n0 = (rem % nt) * GBN;
-    const T *Ab = A + b * p.sAb;
-    const T *Bb = B + b * p.sBb;
+    const int64_t m0 = (rem / nt) * BM, n0 = (rem % nt) * BN;
+    const T *Ab = A + b * p.sAb + m0 * p.sAm;
+    const T *Bb = B + b * p.sBb + n0 * p.sBn;
+    auto load = [&](int64_t ks, int buf) {
+      const int64_t k0 = ks * GBK;
+      gemm_load_side<BM, NT>(Ab + k0 * p.sAk, p.sAm, p.sAk, p.sAk == 1, p.M - m0, p.K - k0,
+                             &As[buf][0][0]);
+      gemm_load_side<BN, NT>(Bb + k0 * p.sBk, p.sBn, p.sBk, p.sBn != 1, p.N - n0, p.K - k0,
+                             &Bs[buf][0][0]);
+    };
     T acc[8][8];
 #pragma unroll
     for (int i = 0; i < 8; ++i)
 #pragma unroll
       for (int j = 0; j < 8; ++j) acc[i][j] = Lim<T>::neg();
     __syncthreads();
-    gemm_load_tile<T>(p, Ab, Bb, m0, n0, 0, &As[0][0][0], &Bs[0][0][0]);
+    load(0, 0);
     cp_async_commit();
     for (int64_t ks = 0; ks < ksteps; ++ks) {
       const int cur = ks & 1;
-      if (ks + 1 < ksteps)
-        gemm_load_tile<T>(p, Ab, Bb, m0, n0, (ks + 1) * GBK, &As[cur ^ 1][0][0], &Bs[cur ^ 1][0][0]);
+      if (ks + 1 < ksteps) load(ks + 1, cur ^ 1);
       cp_async_commit();
       cp_async_wait_prev();
       __syncthreads();
@@ -824,13 +850,13 @@ __global__ void __launch_bounds__(256, 2) k_mpgemm(const GemmParams p, const T *
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
           a0[i] = As[cur][kk][ty * 4 + i];
-          a0[4 + i] = As[cur][kk][64 + ty * 4 + i];
+          a0[4 + i] = As[cur][kk][HM + ty * 4 + i];
           a1[i] = As[cur][kk + 1][ty * 4 + i];
-          a1[4 + i] = As[cur][kk + 1][64 + ty * 4 + i];
+          a1[4 + i] = As[cur][kk + 1][HM + ty * 4 + i];
           b0[i] = Bs[cur][kk][tx * 4 + i];
-          b0[4 + i] = Bs[cur][kk][64 + tx * 4 + i];
+          b0[4 + i] = Bs[cur][kk][HN + tx * 4 + i];
           b1[i] = Bs[cur][kk + 1][tx * 4 + i];
-          b1[4 + i] = Bs[cur][kk + 1][64 + tx * 4 + i];
+          b1[4 + i] = Bs[cur][kk + 1][HN + tx * 4 + i];
         }
 #pragma unroll
         for (int i = 0; i < 8; ++i)
@@ -842,11 +868,11 @@ __global__ void __launch_bounds__(256, 2) k_mpgemm(const GemmParams p, const T *
     T *Cb = C + b * p.sCb;
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
-      const int64_t gm = m0 + (i < 4 ? ty * 4 + i : 64 + ty * 4 + i - 4);
+      const int64_t gm = m0 + (i < 4 ? ty * 4 + i : HM + ty * 4 + i - 4);
       if (gm >= p.M) continue;
 #pragma unroll
       for (int j = 0; j < 8; ++j) {
-        const int64_t gn = n0 + (j < 4 ? tx * 4 + j : 64 + tx * 4 + j - 4);
+        const int64_t gn = n0 + (j < 4 ? tx * 4 + j : HN + tx * 4 + j - 4);
         if (gn < p.N) Cb[gm * p.sCm + gn * p.sCn] = acc[i][j];
       }
     }
@@ -989,7 +1015,7 @@ static int mpgemm16_bn(const GemmParams &p, const void *A, const void *B) {
   return p.N % 128 == 0 ? 128 : p.N % 64 == 0 ? 64 : p.N % 32 == 0 ? 32 : 16;
 }
 
-// ---- tile autotuner.  Candidates: staging (0: 16-byte cp.async, 1: 4-byte)
+// ---- tile autotuner.  Candidates: staging (0: 16-byte cp.async, 1: 4-byte, 2: 4-byte with 64 x 64 tiles)
 // x blocks per SM (2 or 8 of 256 threads).  Every candidate computes each output as
 // the max of the same single-rounding sums, so results are bit-identical and
 // only time decides.  A shape class is timed once, on its first launch
@@ -1047,13 +1073,14 @@ static void tune_store(const std::string &key, GemmTile t) {
 
 // whether a candidate runs on a shape whose widest fast tile is bn (0: none)
 static bool tile_ok(const GemmTile &t, int bn) {
-  return t.per_sm > 0 && (t.variant == 1 || (t.variant == 0 && bn > 0));
+  return t.per_sm > 0 && (t.variant == 1 || t.variant == 2 || (t.variant == 0 && bn > 0));
 }
 
 static cudaError_t run_mpgemm(Dtype dt, const GemmParams &p, const void *A, const void *B, void *C,
                               const Batch &bt, cudaStream_t st, GemmTile t) {
-  int bn = t.variant == 1 ? GBN : mpgemm16_bn(p, A, B);
-  int64_t tiles = p.batch * ((p.M + GBM - 1) / GBM) * ((p.N + bn - 1) / bn);
+  int bn = t.variant == 1 ? GBN : t.variant == 2 ? 64 : mpgemm16_bn(p, A, B);
+  const int bm = t.variant == 2 ? 64 : GBM;
+  int64_t tiles = p.batch * ((p.M + bm - 1) / bm) * ((p.N + bn - 1) / bn);
   if (t.variant == 0 && bn == 128) {
     // 64-wide tiles where they leave the busiest SM less work: a wave's quantum is half
     // as large (2 x 2048^3: 4 tiles of 128 or 7 of 64 on it)
@@ -1076,19 +1103,26 @@ static cudaError_t run_mpgemm(Dtype dt, const GemmParams &p, const void *A, cons
       k_mpgemm16<int32_t, GBM, BN_, 8, TN_, MINB_><<<blocks, (GBM / 8) * (BN_ / TN_), 0, st>>>(  \
           p, (const int32_t *)A, (const int32_t *)B, (int32_t *)C, bt.ib);                       \
   } while (0)
-  if (t.variant != 1) {
+#define TN_MP(BM_, BN_, MINB_)                                                                  \
+  do {                                                                                           \
+    if (dt == DT_F32)                                                                            \
+      k_mpgemm<float, BM_, BN_, MINB_><<<blocks, BM_ * BN_ / 64, 0, st>>>(                       \
+          p, (const float *)A, (const float *)B, (float *)C, bt.ib);                             \
+    else                                                                                         \
+      k_mpgemm<int32_t, BM_, BN_, MINB_><<<blocks, BM_ * BN_ / 64, 0, st>>>(                     \
+          p, (const int32_t *)A, (const int32_t *)B, (int32_t *)C, bt.ib);                       \
+  } while (0)
+  if (t.variant == 0) {
     if (bn == 128) TN_MP16(128, 8, 2);
     else if (bn == 64) TN_MP16(64, 8, 4);
     else if (bn == 32) TN_MP16(32, 4, 6);
     else TN_MP16(16, 2, 8);
+  } else if (t.variant == 2) {
+    TN_MP(64, 64, 8);
   } else {
-    if (dt == DT_F32)
-      k_mpgemm<float><<<blocks, 256, 0, st>>>(p, (const float *)A, (const float *)B, (float *)C,
-                                              bt.ib);
-    else
-      k_mpgemm<int32_t><<<blocks, 256, 0, st>>>(p, (const int32_t *)A, (const int32_t *)B,
-                                                (int32_t *)C, bt.ib);
+    TN_MP(128, 128, 2);
   }
+#undef TN_MP
 #undef TN_MP16
   return cudaGetLastError();
 }
@@ -1291,7 +1325,7 @@ cudaError_t launch_mpgemm(Dtype dt, const GemmParams &p, const void *A, const vo
     if (std::sscanf(f, "%d %d", &t.variant, &t.per_sm) == 2 && tile_ok(t, bn))
       return run_mpgemm(dt, p, A, B, C, bt, st, t);
   }
-  const GemmTile fallback{v16 ? 0 : 1, 8};
+  const GemmTile fallback{v16 ? 0 : tiles * bt.B < num_sms() ? 2 : 1, 8};
   const std::string key = gemm_key(dt, p, bt, v16);
   {
     std::lock_guard<std::mutex> lk(g_tune_mu);
@@ -1306,6 +1340,7 @@ cudaError_t launch_mpgemm(Dtype dt, const GemmParams &p, const void *A, const vo
   std::vector<GemmTile> cand;
   for (int per_sm : {2, 8})   // (the 4-byte kernel loses wherever the 16-byte one applies)
     cand.push_back({v16 ? 0 : 1, per_sm});
+  if (!v16) cand.push_back({2, 8});
   cudaEvent_t e0, e1;
   cudaEventCreate(&e0);
   cudaEventCreate(&e1);

@@ -141,44 +141,6 @@ cudaError_t run_t(bool cnt, const GateSum &p, const SumPtrs &ptr, void *C, uint6
 
 }  // namespace
 
-// The forms: two contracted digits, B a table over (k, n) whose counts are all 1, four or
-// more consecutive outputs (a power of two) per outer index, 32-bit offsets.
-bool gate_sum_leaf(const GateParams &g, bool cnt) {
-  if (g.Ks != 2 || !g.hasB || (cnt && !g.unitB) || g.Ns < 4 || (g.Ns & (g.Ns - 1)) ||
-      g.Ns / 4 > kThreads || !gate_fits32(g))
-    return false;
-  for (int n = 0; n < g.Ns; ++n)
-    if (g.nC[n] != n) return false;
-  for (int s = 0; s < g.nseg; ++s)
-    if (g.seg_sB[s] != 0 || g.seg_sh[s] < 0 || g.seg_sC[s] % 4 != 0) return false;
-  return true;
-}
-
-bool gate_sum_add(GateSum *p, const GateParams &g) {
-  if (p->n == TN_SUM_MAX_G) return false;
-  if (p->n == 0) {
-    p->nseg = g.nseg;
-    p->Ns = g.Ns;
-    p->outer = g.outer;
-    for (int s = 0; s < g.nseg; ++s) {
-      p->seg_size[s] = (int32_t)g.seg_size[s];
-      p->seg_sh[s] = g.seg_sh[s];
-      p->seg_sC[s] = (int32_t)g.seg_sC[s];
-    }
-  }
-  if (p->nseg != g.nseg || p->Ns != g.Ns || p->outer != g.outer) return false;
-  for (int s = 0; s < g.nseg; ++s)
-    if (p->seg_size[s] != g.seg_size[s] || p->seg_sC[s] != g.seg_sC[s]) return false;
-  const int i = p->n++;
-  for (int s = 0; s < g.nseg; ++s) p->seg_sA[i][s] = (int32_t)g.seg_sA[s];
-  for (int k = 0; k < 2; ++k) {
-    p->kA[i][k] = (int32_t)g.kA[k];
-    p->kB[i][k] = (int32_t)g.kB[k];
-  }
-  for (int n = 0; n < g.Ns; ++n) p->nB[i][n] = (int32_t)g.nB[n];
-  return true;
-}
-
 cudaError_t launch_gate_sum(Dtype dt, bool cnt, const GateSum &p, const void *const *A,
                             const void *const *B, const uint64_t *const *nA, void *C,
                             uint64_t *nC, const Batch &bt, cudaStream_t st) {

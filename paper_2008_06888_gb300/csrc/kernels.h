@@ -3,6 +3,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <algorithm>
 #include <vector>
 
 #include "tn_internal.h"
@@ -27,6 +28,27 @@ int num_sms();
 cudaError_t launch_leaves(Dtype dt, int q, const LeafDesc *d_leaves, int nleaves, const float *J,
                           const float *h, char *arena, int P, int rbytes, const Batch &bt,
                           cudaStream_t st);
+
+// whether every outer index (and a grid stride past it) and every element offset of the
+// step fits 32 bits
+inline bool gate_fits32(const GateParams &p) {
+  int64_t a = 0, b = 0, c = 0, ka = 0, kb = 0, nb = 0, nc = 0;
+  for (int s = 0; s < p.nseg; ++s) {
+    a += (p.seg_size[s] - 1) * p.seg_sA[s];
+    b += (p.seg_size[s] - 1) * p.seg_sB[s];
+    c += (p.seg_size[s] - 1) * p.seg_sC[s];
+  }
+  for (int k = 0; k < p.Ks; ++k) {
+    ka = std::max(ka, p.kA[k]);
+    kb = std::max(kb, p.kB[k]);
+  }
+  for (int n = 0; n < p.Ns; ++n) {
+    nb = std::max(nb, p.nB[n]);
+    nc = std::max(nc, p.nC[n]);
+  }
+  const int64_t lim = int64_t(1) << 31;
+  return p.outer < lim / 2 && a + ka < lim && b + kb + nb < lim && c + nc < lim;
+}
 
 // Gate contraction (small B); xA/xB/xC value pointers, nA/nB/nC plane-0
 // pointers (counting only).
@@ -134,8 +156,8 @@ cudaError_t launch_schain(const ChainParams &p, const char *arena, const void *A
                           cudaStream_t st);
 
 // Sum of n = 2 or 4 gate contractions over the same output indices (gate_sum.cu):
-// n = 2: G0 + G1, n = 4: (G0 + G1) + (G2 + G3); counts multiply.  gate_sum_leaf: whether
-// a gate has the form it takes; gate_sum_add: append one (false: its outputs differ).
+// n = 2: G0 + G1, n = 4: (G0 + G1) + (G2 + G3); counts multiply (the forms it takes:
+// gate_sum_leaf in program.cpp).
 constexpr int TN_SUM_MAX_G = 4;
 struct GateSum {
   int32_t n = 0, nseg = 0, Ns = 0;
@@ -144,8 +166,6 @@ struct GateSum {
   int32_t seg_sA[TN_SUM_MAX_G][TN_MAX_SEG];
   int32_t kA[TN_SUM_MAX_G][2], kB[TN_SUM_MAX_G][2], nB[TN_SUM_MAX_G][TN_GATE_MAX_N];
 };
-bool gate_sum_leaf(const GateParams &g, bool cnt);
-bool gate_sum_add(GateSum *p, const GateParams &g);
 cudaError_t launch_gate_sum(Dtype dt, bool cnt, const GateSum &p, const void *const *A,
                             const void *const *B, const uint64_t *const *nA, void *C,
                             uint64_t *nC, const Batch &bt, cudaStream_t st);

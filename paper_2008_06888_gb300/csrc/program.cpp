@@ -1471,8 +1471,9 @@ struct Builder {
     // integral counts without folding have no register-chain kernel
     if (pr.sat && !folded() && pr.dt == DT_I32) regmode = false;
     // q = 3 tiles: 8 legs (26 KB, two of them staged per block, four blocks per SM) of
-    // which 4 are the fastest, for runs of 81 elements; 7 with the counts' planes
-    if (q == 3) { tmax = P == 0 ? 8 : 7; wlow = 4; }
+    // which 4 are the fastest, for runs of 81 elements; 7 with the counts' planes, and
+    // where programs are only scored (the order search ranks orders as it always has)
+    if (q == 3) { tmax = P == 0 && small_runs ? 8 : 7; wlow = 4; }
     emit_leaves();
     if (!forward()) return false;
     pr.root = loc[plan.root];

@@ -769,6 +769,17 @@ struct Builder {
     return T;
   }
 
+  // legs of a chain's tiles: the local set, for q = 3 values filled up with the fastest
+  // other legs (k_chain3 gives every 27 elements of a tile a thread, so a small tile
+  // leaves most of a block idle: a 3^15 chain with two slow legs took 142 us)
+  std::vector<int> tile_legs(int R, const std::vector<int> &touched) const {
+    std::vector<int> T = local_set(R, touched);
+    for (int p = R - 1; q == 3 && P == 0 && p >= 0 && (int)T.size() < tmax; --p)
+      if (pos_of(T, p) < 0) T.push_back(p);
+    std::sort(T.begin(), T.end());
+    return T;
+  }
+
   bool fits(const Macro &m, const CGate &g) const {
     if ((int)m.gates.size() >= TN_CHAIN_MAX_G) return false;
     if (regmode) {
@@ -929,7 +940,7 @@ struct Builder {
     ChainParams cp{};
     const std::vector<int> &ord = order[m.out];
     const int R = (int)ord.size();
-    std::vector<int> T = local_set(R, m.touched);
+    std::vector<int> T = tile_legs(R, m.touched);
     cp.q = q;
     cp.t = (int)T.size();
     cp.tile = (int)ipow(q, cp.t);
@@ -1135,7 +1146,7 @@ struct Builder {
         // input (without the grown leg, if any)
         const std::vector<int> &ord = m.state.empty() ? order[m.out] : m.state;
         const int R = (int)ord.size();
-        std::vector<int> T = regmode ? reg_legs(m) : local_set(R, m.touched);
+        std::vector<int> T = regmode ? reg_legs(m) : tile_legs(R, m.touched);
         for (int p = 0; p < R; ++p) {
           if (pos_of(T, p) >= 0) continue;
           ct.out_spin[ct.nout] = ord[p];

@@ -750,7 +750,6 @@ def run_sample(args):
                                "probability from exact counts (3 primes + witness)",
                    "log2_peak_elements": sg.log2_peak},
         "ground_states": str(count), "E_min": E, "distinct_in_last_call": distinct,
-        "count_calls_per_call": inst["n"] + 1, "instances_per_count_call": 2 * S,
         "ms_per_call": dt * 1e3}), flush=True)
 
 

@@ -6,7 +6,7 @@
 // 108 us for a 15 x 15 lattice (7.0 ms), where moving the 3^15 elements takes 17 us.  Here the gates are cut into groups
 // of at most three replaced legs: a thread holds the 27 elements that differ in a group's
 // legs in registers, applies all of its gates there and writes them back, so a chain
-// makes two or three passes over its tile (46 chains of 57 us, 2.6 ms).  Gates on other legs of the tile read the
+// makes two or three passes over its tile (46 chains of 52 us, 2.4 ms).  Gates on other legs of the tile read the
 // thread's fixed digits.  Blocks are persistent and copy the next tile (cp.async) while
 // they work on this one.
 // Every element sees the same sums and maxima in the same order as one gate at a time.

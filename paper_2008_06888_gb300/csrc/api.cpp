@@ -956,8 +956,15 @@ tn_status tn_set_couplings(tn_ctx *ctx, const float *J, const float *h, int32_t 
 
 tn_status tn_set_stream(tn_ctx *ctx, void *cuda_stream) {
   if (!ctx) return TN_EINVAL;
-  if (ctx->up_pending) CK(cudaEventSynchronize(ctx->up_ev));
-  ctx->up_pending = false;
+  if (ctx->up_pending) {
+    // relaxed: the event is no part of a capture that this thread may have in progress
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    CK(cudaThreadExchangeStreamCaptureMode(&mode));
+    const cudaError_t e = cudaEventSynchronize(ctx->up_ev);
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    CK(e);
+    ctx->up_pending = false;
+  }
   ctx->stream = (cudaStream_t)cuda_stream;
   return TN_OK;
 }

@@ -35,3 +35,20 @@ def test_changes_reach_the_next_call(fields):
         sg.set_stream(streams[k % 2].cuda_stream)
         assert sg.energy() == ref.energy()
         assert sg.count(3) == ref.count(3)
+
+
+def test_stream_change_inside_a_capture():
+    """tn_set_stream after an upload leaves a capture of the caller's work alone."""
+    inst = I.square_lattice(6, coupling="pm1", seed=2)
+    sg = P.SpinGlass(inst, order="sweep", seq=I.square_sweep_order(6))
+    E = sg.energy()
+    x = torch.zeros(8, device="cuda")
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, capture_error_mode="global"):
+        sg.set_stream(torch.cuda.current_stream().cuda_stream)
+        x += 1
+    g.replay()
+    torch.cuda.synchronize()
+    sg.set_stream(0)
+    assert float(x.sum()) == 8.0 and sg.energy() == E

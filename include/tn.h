@@ -135,7 +135,8 @@ int32_t tn_leaf_count(const tn_ctx *ctx);
 
 /*
  * tn_set_couplings -- replace J (n_edges) and h (n_spins, or NULL = keep)
- *   without re-planning.  on_device = 0: host pointers (copied synchronously);
+ *   without re-planning.  on_device = 0: host pointers, copied before the call
+ *   returns (it waits for an upload of earlier host values that is still queued);
  *   1: device pointers on the context's device (copied on the context stream).
  *   INT32 contexts require integral values (TN_EINVAL otherwise, host only).
  */

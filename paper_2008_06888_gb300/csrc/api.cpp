@@ -156,6 +156,19 @@ void free_program(Program *p) {
   p->d_chain_traces = nullptr;
 }
 
+// Waits until the last upload of host couplings has read them.
+tn_status wait_upload(tn_ctx *ctx) {
+  if (!ctx->up_pending) return TN_OK;
+  // relaxed: the event is no part of a capture that this thread may have in progress
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  CK(cudaThreadExchangeStreamCaptureMode(&mode));
+  const cudaError_t e = cudaEventSynchronize(ctx->up_ev);
+  cudaThreadExchangeStreamCaptureMode(&mode);
+  CK(e);
+  ctx->up_pending = false;
+  return TN_OK;
+}
+
 tn_status ensure_device(tn_ctx *ctx) {
   if (!ctx->dev_ready) {
     int ndev = 0;
@@ -191,9 +204,11 @@ tn_status ensure_device(tn_ctx *ctx) {
     if (n.m)
       CK(cudaMemcpyAsync(ctx->d_J, n.J.data(), n.m * sizeof(float), cudaMemcpyHostToDevice,
                          ctx->stream));
-    // Pageable sources: the calls return once the values are staged, and what uses them
-    // follows on the same stream (tn_set_stream waits for the event), so nothing waits
-    // here.  An instance without fields keeps the zeros written when its buffers were made.
+    // The copies may read net.J and net.h after the calls have returned (a host whose page
+    // tables the device shares need not stage them), and what uses the values follows on
+    // the same stream: nothing waits here, and whoever changes or frees those arrays or
+    // takes another stream waits for the event first (wait_upload).  An instance without
+    // fields keeps the zeros written when its buffers were made.
     // (6x6 energy + count: 111 -> 95 us with this and one result copy of a count.)
     if (!n.h.empty())
       CK(cudaMemcpyAsync(ctx->d_h, n.h.data(), n.n * sizeof(float), cudaMemcpyHostToDevice,
@@ -939,6 +954,8 @@ tn_status tn_set_couplings(tn_ctx *ctx, const float *J, const float *h, int32_t 
     if (h) nh.assign(h, h + n.n);
     if (ctx->dt == DT_I32 && !(integral(nj) && integral(nh)))
       return fail(ctx, TN_EINVAL, "INT32 context needs integral J, h");
+    const tn_status s = wait_upload(ctx);
+    if (s != TN_OK) return s;
     n.J = nj;
     n.h = nh;
     ctx->couplings_dirty = true;
@@ -956,15 +973,8 @@ tn_status tn_set_couplings(tn_ctx *ctx, const float *J, const float *h, int32_t 
 
 tn_status tn_set_stream(tn_ctx *ctx, void *cuda_stream) {
   if (!ctx) return TN_EINVAL;
-  if (ctx->up_pending) {
-    // relaxed: the event is no part of a capture that this thread may have in progress
-    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
-    CK(cudaThreadExchangeStreamCaptureMode(&mode));
-    const cudaError_t e = cudaEventSynchronize(ctx->up_ev);
-    cudaThreadExchangeStreamCaptureMode(&mode);
-    CK(e);
-    ctx->up_pending = false;
-  }
+  const tn_status s = wait_upload(ctx);
+  if (s != TN_OK) return s;
   ctx->stream = (cudaStream_t)cuda_stream;
   return TN_OK;
 }
@@ -1925,6 +1935,7 @@ const char *tn_last_error(const tn_ctx *ctx) {
 
 void tn_destroy(tn_ctx *ctx) {
   if (!ctx) return;
+  wait_upload(ctx);
   for (auto &p : ctx->prog) if (p) free_program(p.get());
   if (ctx->prog_pass) free_program(ctx->prog_pass.get());
   if (ctx->prog_sat) free_program(ctx->prog_sat.get());

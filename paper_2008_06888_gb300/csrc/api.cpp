@@ -169,6 +169,13 @@ tn_status wait_upload(tn_ctx *ctx) {
   return TN_OK;
 }
 
+// Waits for the context's stream, and so for an upload queued on it.
+cudaError_t wait_stream(tn_ctx *ctx) {
+  const cudaError_t e = cudaStreamSynchronize(ctx->stream);
+  if (e == cudaSuccess) ctx->up_pending = false;
+  return e;
+}
+
 tn_status ensure_device(tn_ctx *ctx) {
   if (!ctx->dev_ready) {
     int ndev = 0;
@@ -704,7 +711,7 @@ tn_status batch_roots(tn_ctx *ctx, const Program &p, int B, std::vector<char> *r
 tn_status check_trace_err(tn_ctx *ctx) {
   int herr = 0;
   CK(cudaMemcpyAsync(&herr, ctx->d_err, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
-  CK(cudaStreamSynchronize(ctx->stream));
+  CK(wait_stream(ctx));
   if (herr) {
     cudaMemsetAsync(ctx->d_err, 0, sizeof(int), ctx->stream);
     return fail(ctx, TN_EINVAL, "traceback met an unassigned spin (internal planning error)");
@@ -991,7 +998,7 @@ tn_status tn_energy(tn_ctx *ctx, double *E) {
   char raw[4];
   CK(cudaMemcpyAsync(raw, ctx->d_arena + abs_off(*p, p->root), 4, cudaMemcpyDeviceToHost,
                      ctx->stream));
-  CK(cudaStreamSynchronize(ctx->stream));
+  CK(wait_stream(ctx));
   *E = root_energy(ctx, raw);
   return TN_OK;
 }
@@ -1009,7 +1016,7 @@ tn_status tn_forward(tn_ctx *ctx, double *E) {
     char raw[4];
     CK(cudaMemcpyAsync(raw, ctx->d_arena + abs_off(*p, p->root), 4, cudaMemcpyDeviceToHost,
                        ctx->stream));
-    CK(cudaStreamSynchronize(ctx->stream));
+    CK(wait_stream(ctx));
     *E = root_energy(ctx, raw);
   }
   ctx->fwd_done = true;
@@ -1027,7 +1034,7 @@ tn_status tn_backward(tn_ctx *ctx, int8_t *sigma) {
   if ((s = run_program(ctx, p, p.fwd_end, (int)p.ops.size())) != TN_OK) return s;
   int herr = 0;
   CK(cudaMemcpyAsync(&herr, ctx->d_err, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
-  CK(cudaStreamSynchronize(ctx->stream));
+  CK(wait_stream(ctx));
   if (herr) {
     cudaMemsetAsync(ctx->d_err, 0, sizeof(int), ctx->stream);
     return fail(ctx, TN_EINVAL, "traceback met an unassigned spin (internal planning error)");
@@ -1037,7 +1044,7 @@ tn_status tn_backward(tn_ctx *ctx, int8_t *sigma) {
     CK(launch_state_out(ctx->net.q, ctx->net.n, ctx->d_state, ctx->d_out, 1, ctx->stream));
     ctx->launches[5]++;
     CK(cudaMemcpyAsync(sigma, ctx->d_out, ctx->net.n, cudaMemcpyDeviceToHost, ctx->stream));
-    CK(cudaStreamSynchronize(ctx->stream));
+    CK(wait_stream(ctx));
   }
   return TN_OK;
 }
@@ -1063,7 +1070,7 @@ tn_status tn_gradient(tn_ctx *ctx, float *dJ, float *dh, int32_t on_device) {
   CK(launch_grad(n.q, n.n, n.m, ctx->d_eu, ctx->d_ev, ctx->d_state, gJ, gh, 1, ctx->stream));
   if (dJ && n.m) CK(cudaMemcpyAsync(dJ, gJ, n.m * sizeof(float), cudaMemcpyDeviceToHost, ctx->stream));
   if (dh) CK(cudaMemcpyAsync(dh, gh, n.n * sizeof(float), cudaMemcpyDeviceToHost, ctx->stream));
-  CK(cudaStreamSynchronize(ctx->stream));
+  CK(wait_stream(ctx));
   cudaFree(gJ);
   cudaFree(gh);
   return TN_OK;
@@ -1093,7 +1100,7 @@ tn_status tn_count(tn_ctx *ctx, int32_t n_primes, uint64_t *limbs, int32_t *n_li
       std::vector<char> raw(p->root.noff + 8 - p->root.xoff);
       CK(cudaMemcpyAsync(raw.data(), base + p->root.xoff, raw.size(), cudaMemcpyDeviceToHost,
                          ctx->stream));
-      CK(cudaStreamSynchronize(ctx->stream));
+      CK(wait_stream(ctx));
       std::memcpy(&v, raw.data() + raw.size() - 8, 8);
       if (v < kSaturated) {
         if (E) *E = root_energy(ctx, raw.data());
@@ -1117,7 +1124,7 @@ tn_status tn_count(tn_ctx *ctx, int32_t n_primes, uint64_t *limbs, int32_t *n_li
   for (int i = 0; i < rep.P; ++i)   // little-endian: a 4-byte residue fills the low half
     CK(cudaMemcpyAsync(&res[i], base + p->root.noff + (int64_t)i * p->root.plane * rep.rb, rep.rb,
                        cudaMemcpyDeviceToHost, ctx->stream));
-  CK(cudaStreamSynchronize(ctx->stream));
+  CK(wait_stream(ctx));
   if (E) *E = root_energy(ctx, raw);
   return finish_count(ctx, res, rep.primes, limbs, n_limbs, ln_count);
 }
@@ -1185,7 +1192,7 @@ tn_status count_in_passes(tn_ctx *ctx, int n_primes, uint64_t *limbs, int32_t *n
     uint32_t r = 0;
     if (j == 0) CK(cudaMemcpyAsync(raw, base + p.root.xoff, 4, cudaMemcpyDeviceToHost, ctx->stream));
     CK(cudaMemcpyAsync(&r, base + p.root.noff, 4, cudaMemcpyDeviceToHost, ctx->stream));
-    CK(cudaStreamSynchronize(ctx->stream));
+    CK(wait_stream(ctx));
     res[j] = r;
   }
   if (E) *E = root_energy(ctx, raw);
@@ -1209,7 +1216,7 @@ tn_status tn_energy_batch(tn_ctx *ctx, int32_t B, const float *J, const float *h
   if ((s = run_program(ctx, *p, 0, -1, ra)) != TN_OK) return s;
   std::vector<char> raw;
   if ((s = batch_roots(ctx, *p, B, &raw)) != TN_OK) return s;
-  CK(cudaStreamSynchronize(ctx->stream));
+  CK(wait_stream(ctx));
   for (int b = 0; b < B; ++b) E[b] = root_energy(ctx, raw.data() + 4 * b);
   return TN_OK;
 }
@@ -1378,7 +1385,7 @@ tn_status tn_count_batch(tn_ctx *ctx, int32_t B, const float *J, const float *h,
   std::vector<char> raw((size_t)B * 4);
   std::vector<uint64_t> res((size_t)P * B);
   if ((s = stage_results(ctx, *p, B, P, raw.data(), res.data())) != TN_OK) return s;
-  CK(cudaStreamSynchronize(ctx->stream));
+  CK(wait_stream(ctx));
   std::vector<int32_t> own(status ? 0 : B, TN_OK);
   if (!status) status = own.data();
   s = finish_counts(ctx, B, rep, raw.data(), res.data(), limbs, limbs_per, E, status, sat);
@@ -1837,7 +1844,7 @@ tn_status sample_by_frontier(tn_ctx *ctx, const std::vector<int> &order,
   CK(cudaMemcpyAsync(&total, d + oN, 8, cudaMemcpyDeviceToHost, ctx->stream));
   CK(cudaMemcpyAsync(out.data(), d + oG, out.size(), cudaMemcpyDeviceToHost, ctx->stream));
   CK(cudaMemcpyAsync(&herr, ctx->d_err, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
-  CK(cudaStreamSynchronize(ctx->stream));
+  CK(wait_stream(ctx));
   if (herr) CK(cudaMemsetAsync(ctx->d_err, 0, sizeof(int), ctx->stream));
   if (ctx->sample_cap > kSampleKeep) {
     CK(cudaFree(ctx->d_sample));

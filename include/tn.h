@@ -187,7 +187,12 @@ tn_status tn_gradient(tn_ctx *ctx, float *dJ, float *dh, int32_t on_device);
 /*
  * tn_count -- ground-state degeneracy with the counting tuples of Sec. II.
  *   n_primes in [1, 8] sets the range: the count is exact up to about
- *   2^(61*n_primes).  The residues are kept modulo ceil(61*n_primes/31)
+ *   2^(61*n_primes).  Counts below 2^59 need no residues: the first run keeps
+ *   one 8-byte plane of exact, saturating counts, and only a count that
+ *   reaches 2^59 there is run again with residue planes.  A context whose last
+ *   counts did starts with the residues, until its counts are small again
+ *   (before its first count the number of spins decides); TN_COUNT_RESIDUES
+ *   leaves the saturating run out.  The residues are kept modulo ceil(61*n_primes/31)
  *   31-bit primes 2^31 - c in 4-byte planes when those fit in 9 planes
  *   (n_primes <= 4; TN_COUNT_61 forces the other form), else modulo n_primes
  *   61-bit primes 2^61 - c in 8-byte planes; one extra witness prime checks
@@ -235,10 +240,11 @@ tn_status tn_sample(tn_ctx *ctx, int32_t n_samples, uint64_t seed, const int32_t
  * tn_config_batch -- E_min and the ground state (sigma: B*n_spins int8, host,
  *   may be NULL; same conventions as tn_config).
  * tn_count_batch -- E_min and degeneracy of each instance with the range of
- *   n_primes 61-bit primes + witness (residue planes as tn_count); limbs:
- *   B*limbs_per little-endian 64-bit limbs; status[b] (may be NULL) is TN_OK,
- *   TN_EOVERFLOW or TN_EINVAL (count needs more than limbs_per limbs).
- *   Returns the first non-OK status.
+ *   n_primes 61-bit primes + witness (planes as tn_count: instances that
+ *   saturate are run again as a batch of their own); limbs: B*limbs_per
+ *   little-endian 64-bit limbs; status[b] (may be NULL) is TN_OK, TN_EOVERFLOW
+ *   or TN_EINVAL (count needs more than limbs_per limbs).  Returns the first
+ *   non-OK status.
  */
 tn_status tn_energy_batch(tn_ctx *ctx, int32_t B, const float *J, const float *h,
                           int32_t on_device, double *E);

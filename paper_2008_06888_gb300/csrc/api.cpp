@@ -53,6 +53,7 @@ struct tn_ctx {
   int64_t arena_cap = 0;
   std::unique_ptr<Program> prog[3];
   std::unique_ptr<Program> prog_sat;   // counts in one plane of exact 64-bit integers
+  int big_counts = -1;   // whether counts start with residues: -1 by size, else as the last did
   int prog_P = 0, prog_rb = 8;
   bool have_state = false;
   bool fwd_done = false;   // tn_forward ran last; its checkpoints are live
@@ -747,19 +748,37 @@ CountRep count_rep(int n_primes) {
 // Counts below 2^59 need no residues: one 8-byte plane holds them exactly,
 // 4 + 8 bytes per element instead of 4 + 28 (mixed +-J batches of side 8..20: 192
 // instances in 15.0 ms instead of 46.6), and saturates where they do not fit; such an
-// instance is run again with the residue planes.  Contexts whose counts are likely to
-// be larger start there: +-J glasses have up to about 0.105 bits of ground-state
-// entropy per spin without fields (square lattices; 3-regular and chimera graphs less),
-// Max-2-SAT formulas about 0.35 bits per variable, so 59 bits hold up to some 540 spins
-// without and 165 with fields.  TN_COUNT_RESIDUES keeps the residue planes.
-bool sat_first(const tn_ctx *ctx) {
+// instance is run again with the residue planes.  A context goes by its last counts
+// (note_counts).  Before it has any: +-J glasses have up to about 0.105 bits of
+// ground-state entropy per spin without fields (square lattices; 3-regular and chimera
+// graphs less), Max-2-SAT formulas about 0.35 bits per variable, so 59 bits hold up to
+// some 540 spins without and 165 with fields.  TN_COUNT_RESIDUES keeps the residue planes.
+bool residues_forced() {
   for (const char *v : {"TN_COUNT_RESIDUES", "TN_COUNT_61", "TN_COUNT_PASSES"})
-    if (std::getenv(v)) return false;
+    if (std::getenv(v)) return true;
+  return false;
+}
+bool sat_first(const tn_ctx *ctx) {
+  if (residues_forced()) return false;
+  if (ctx->big_counts >= 0) return !ctx->big_counts;
   return ctx->net.n <= (ctx->net.h.empty() ? 540 : 165) || ctx->dt == DT_F32;
 }
 // an exact count stays below this; one at or above it may have saturated (the chain
 // kernel's cap, chain_sat.cu)
 constexpr uint64_t kSaturated = 1ull << 59;
+
+// How the next counts start when `big` of the last B reached 2^59: with residues where
+// those for all B cost less than the saturating run and residues for `big` instances.  An
+// element costs about three times as much in a residue step, and a saturating step's latency
+// (2.5 us) is the time of 2^19 elements, so that is (3 - 1) B - 3 big elements' work below
+// 2^19.  (16 lattices of side 14, 4 or 8 of them big: 0.92 ms with residues at once, 1.27
+// with two runs; side 20, 8 big: 24.4 and 20.7; 134 lattices of side 8 to 20, 2 of them
+// big: 35.0 and 12.4.)
+void note_counts(tn_ctx *ctx, int big, int B) {
+  ctx->big_counts =
+      big > 0 && (2.0 * B - 3.0 * big) * std::exp2(ctx->plan.log2_peak) < (double)(1 << 19);
+}
+bool is_big(const std::vector<uint64_t> &limbs) { return limbs.size() > 1 || limbs[0] >= kSaturated; }
 
 // exact count from residues res[i] modulo rep.primes[i] (the last one the witness)
 tn_status count_from_residues(tn_ctx *ctx, const std::vector<uint64_t> &res, const CountRep &rep,
@@ -1140,7 +1159,9 @@ tn_status finish_count(tn_ctx *ctx, const std::vector<uint64_t> &res,
   const size_t n = pr.size() - 1;
   std::vector<uint64_t> r(res.begin(), res.begin() + n), p(pr.begin(), pr.begin() + n);
   std::vector<uint64_t> v = crt(r, p);
-  if (limbs_mod(v, pr[n]) != res[n])
+  const bool fits = limbs_mod(v, pr[n]) == res[n];
+  note_counts(ctx, !fits || is_big(v), 1);
+  if (!fits)
     return fail(ctx, TN_EOVERFLOW, "count exceeds the product of the primes (witness mismatch)");
   if (n_limbs) {
     if (limbs && *n_limbs < (int32_t)v.size())
@@ -1284,19 +1305,25 @@ tn_status pinned_stage(tn_ctx *ctx, size_t bytes, char **out) {
 
 // E, counts and statuses of B instances from their staged root values (raw:
 // 4 bytes each) and residues (res[i * B + b], plane i, the last the witness) or, with
-// sat, exact counts (res[b]; saturated instances are left out).
+// sat, exact counts (res[b]; saturated instances are left out).  *big: the number of
+// counts of 2^59 and more.
 tn_status finish_counts(tn_ctx *ctx, int B, const CountRep &rep, const char *raw,
                         const uint64_t *res, uint64_t *limbs, int32_t limbs_per, double *E,
-                        int32_t *status, bool sat = false) {
+                        int32_t *status, int *big, bool sat = false) {
   const int P = rep.P;
   tn_status first = TN_OK;
+  *big = 0;
   for (int b = 0; b < B; ++b) {
-    if (sat && res[b] >= kSaturated) continue;
+    if (sat && res[b] >= kSaturated) {
+      ++*big;
+      continue;
+    }
     if (E) E[b] = root_energy(ctx, raw + 4 * b);
     std::vector<uint64_t> r(P), v;
     if (sat) r = residues_of(res[b], rep);
     else for (int i = 0; i < P; ++i) r[i] = res[(size_t)i * B + b];
     tn_status sb = count_from_residues(ctx, r, rep, &v);
+    if (sb != TN_OK || is_big(v)) ++*big;
     if (sb == TN_OK && (int)v.size() > limbs_per) {
       sb = TN_EINVAL;
       fail(ctx, sb, "limbs_per too small for a count");
@@ -1310,6 +1337,19 @@ tn_status finish_counts(tn_ctx *ctx, int B, const CountRep &rep, const char *raw
 }
 
 tn_status stage_results(tn_ctx *ctx, const Program &p, int B, int P, char *raw, uint64_t *res);
+
+// batch_setup of the program that counts of B instances start with.  Residues that earlier
+// counts asked for but whose planes do not fit for all B give way to the saturating run.
+tn_status count_setup(tn_ctx *ctx, int B, const float *J, const float *h, int on_device,
+                      const CountRep &rep, bool *sat, Program **p, RunArgs *ra) {
+  *sat = sat_first(ctx);
+  if (!*sat) {
+    const tn_status s = batch_setup(ctx, B, J, h, on_device, PM_COUNT, rep.P, p, ra, rep.rb);
+    if (s != TN_ENOMEM || residues_forced() || ctx->big_counts != 1) return s;
+    *sat = true;
+  }
+  return batch_setup(ctx, B, J, h, on_device, PM_COUNT, 1, p, ra, 8, true);
+}
 
 // E, counts and statuses of the instances ids[0..K) of a batch (arrays of the whole
 // batch), counted with the residue planes of `rep`.  Returns whether the run itself
@@ -1330,8 +1370,10 @@ tn_status count_residues(tn_ctx *ctx, const std::vector<int> &ids, const float *
     s = fail(ctx, TN_ECUDA, "counting with residue planes failed");
   std::vector<double> Ek(K);
   std::vector<int32_t> sk(K, s);
+  int big = 0;
   if (s == TN_OK)
-    finish_counts(ctx, K, rep, raw.data(), res.data(), lk.data(), limbs_per, Ek.data(), sk.data());
+    finish_counts(ctx, K, rep, raw.data(), res.data(), lk.data(), limbs_per, Ek.data(), sk.data(),
+                  &big);
   for (int k = 0; k < K; ++k) {
     std::copy(lk.begin() + (size_t)k * limbs_per, lk.begin() + (size_t)(k + 1) * limbs_per,
               limbs + (int64_t)ids[k] * limbs_per);
@@ -1375,12 +1417,12 @@ tn_status tn_count_batch(tn_ctx *ctx, int32_t B, const float *J, const float *h,
     return fail(ctx, TN_EINVAL, "n_primes must be in [1, 8]");
   if (!limbs || limbs_per < 1) return fail(ctx, TN_EINVAL, "limbs buffer missing");
   const CountRep rep = count_rep(n_primes);
-  const bool sat = sat_first(ctx);
-  const int P = sat ? 1 : rep.P;
+  bool sat = false;
   Program *p;
   RunArgs ra;
-  tn_status s = batch_setup(ctx, B, J, h, on_device, PM_COUNT, P, &p, &ra, sat ? 8 : rep.rb, sat);
+  tn_status s = count_setup(ctx, B, J, h, on_device, rep, &sat, &p, &ra);
   if (s != TN_OK) return s;
+  const int P = sat ? 1 : rep.P;
   if ((s = run_program(ctx, *p, 0, -1, ra)) != TN_OK) return s;
   std::vector<char> raw((size_t)B * 4);
   std::vector<uint64_t> res((size_t)P * B);
@@ -1388,7 +1430,9 @@ tn_status tn_count_batch(tn_ctx *ctx, int32_t B, const float *J, const float *h,
   CK(wait_stream(ctx));
   std::vector<int32_t> own(status ? 0 : B, TN_OK);
   if (!status) status = own.data();
-  s = finish_counts(ctx, B, rep, raw.data(), res.data(), limbs, limbs_per, E, status, sat);
+  int big = 0;
+  s = finish_counts(ctx, B, rep, raw.data(), res.data(), limbs, limbs_per, E, status, &big, sat);
+  note_counts(ctx, big, B);
   std::vector<int> over;
   for (int b = 0; sat && b < B; ++b)
     if (res[b] >= kSaturated) over.push_back(b);
@@ -1505,7 +1549,6 @@ tn_status tn_batch_run(int32_t B, tn_ctx *const *ctxs, double *E, uint64_t *limb
     off += (size_t)G * 8 * P;
     r.raw = stage + off;
     off += ((size_t)G * 4 + 63) / 64 * 64;
-    r.sat = limbs && sat_first(r.owner);
     std::vector<float> &J = r.J, &h = r.h;
     J.resize((size_t)G * n.m);
     h.resize(n.h.empty() ? 0 : (size_t)G * n.n);
@@ -1526,9 +1569,9 @@ tn_status tn_batch_run(int32_t B, tn_ctx *const *ctxs, double *E, uint64_t *limb
     }
     r.owner->stream = st;
     RunArgs ra;
-    r.s = batch_setup(r.owner, G, J.data(), h.empty() ? nullptr : h.data(), 0,
-                      limbs ? PM_COUNT : PM_ENERGY, r.sat ? 1 : P, &r.p, &ra,
-                      r.sat ? 8 : rep.rb, r.sat);
+    const float *hp = h.empty() ? nullptr : h.data();
+    r.s = limbs ? count_setup(r.owner, G, J.data(), hp, 0, rep, &r.sat, &r.p, &ra)
+                : batch_setup(r.owner, G, J.data(), hp, 0, PM_ENERGY, 0, &r.p, &ra);
     if (r.s == TN_OK) r.s = run_program(r.owner, *r.p, 0, -1, ra);
     if (r.s == TN_OK) r.s = stage_results(r.owner, *r.p, G, r.sat ? 1 : P, r.raw, r.res);
   }
@@ -1548,8 +1591,10 @@ tn_status tn_batch_run(int32_t B, tn_ctx *const *ctxs, double *E, uint64_t *limb
     tn_status s = r.s;
     if (s == TN_OK && limbs) {
       std::vector<uint64_t> lg((size_t)G * limbs_per);
+      int big = 0;
       s = finish_counts(r.owner, G, rep, r.raw, r.res, lg.data(), limbs_per, Eg.data(), sg.data(),
-                        r.sat);
+                        &big, r.sat);
+      note_counts(r.owner, big, G);
       std::vector<int> over;
       for (int g = 0; r.sat && g < G; ++g)
         if (r.res[g] >= kSaturated) over.push_back(g);
@@ -1801,8 +1846,7 @@ tn_status sample_by_frontier(tn_ctx *ctx, const std::vector<int> &order,
                              const std::vector<float> &h, int S, uint64_t seed, int8_t *sigma,
                              bool *done) {
   *done = false;
-  for (const char *v : {"TN_COUNT_RESIDUES", "TN_COUNT_61", "TN_COUNT_PASSES"})
-    if (std::getenv(v)) return TN_OK;
+  if (residues_forced()) return TN_OK;
   const Net &n = ctx->net;
   FrontierPlan fp;
   if (!plan_frontier(n.n, n.eu, n.ev, n.J, h, order, 26, &fp)) return TN_OK;

@@ -1351,29 +1351,34 @@ tn_status count_setup(tn_ctx *ctx, int B, const float *J, const float *h, int on
   return batch_setup(ctx, B, J, h, on_device, PM_COUNT, 1, p, ra, 8, true);
 }
 
-// E, counts and statuses of the instances ids[0..K) of a batch (arrays of the whole
-// batch), counted with the residue planes of `rep`.  Returns whether the run itself
-// worked (else its error is their status).
-tn_status count_residues(tn_ctx *ctx, const std::vector<int> &ids, const float *J, const float *h,
-                         int on_device, const CountRep &rep, uint64_t *limbs, int32_t limbs_per,
-                         double *E, int32_t *status) {
+// Queues the residue planes' count of the instances ids[0..K) of a batch (J, h: arrays of
+// the whole batch) and the copies of its results to raw (4 K bytes) and res (rep.P K words).
+tn_status queue_residues(tn_ctx *ctx, const std::vector<int> &ids, const float *J, const float *h,
+                         int on_device, const CountRep &rep, char *raw, uint64_t *res) {
   const int K = (int)ids.size();
   Program *p;
   RunArgs ra;
   tn_status s = batch_setup(ctx, K, J, h, on_device, PM_COUNT, rep.P, &p, &ra, rep.rb, false,
                             ids.data());
   if (s == TN_OK) s = run_program(ctx, *p, 0, -1, ra);
-  std::vector<char> raw((size_t)K * 4);
-  std::vector<uint64_t> res((size_t)rep.P * K), lk((size_t)K * limbs_per);
-  if (s == TN_OK) s = stage_results(ctx, *p, K, rep.P, raw.data(), res.data());
-  if (s == TN_OK && cudaStreamSynchronize(ctx->stream) != cudaSuccess)
+  return s == TN_OK ? stage_results(ctx, *p, K, rep.P, raw, res) : s;
+}
+
+// Waits for that count (s: the status of its queuing) and files E, counts and statuses
+// with those of the batch.  Returns whether the run itself worked (else its error is the
+// instances' status).
+tn_status finish_residues(tn_ctx *ctx, tn_status s, const std::vector<int> &ids,
+                          const CountRep &rep, const char *raw, const uint64_t *res,
+                          uint64_t *limbs, int32_t limbs_per, double *E, int32_t *status) {
+  const int K = (int)ids.size();
+  const cudaError_t e = cudaStreamSynchronize(ctx->stream);
+  if (s == TN_OK && e != cudaSuccess)
     s = fail(ctx, TN_ECUDA, "counting with residue planes failed");
+  std::vector<uint64_t> lk((size_t)K * limbs_per);
   std::vector<double> Ek(K);
   std::vector<int32_t> sk(K, s);
   int big = 0;
-  if (s == TN_OK)
-    finish_counts(ctx, K, rep, raw.data(), res.data(), lk.data(), limbs_per, Ek.data(), sk.data(),
-                  &big);
+  if (s == TN_OK) finish_counts(ctx, K, rep, raw, res, lk.data(), limbs_per, Ek.data(), sk.data(), &big);
   for (int k = 0; k < K; ++k) {
     std::copy(lk.begin() + (size_t)k * limbs_per, lk.begin() + (size_t)(k + 1) * limbs_per,
               limbs + (int64_t)ids[k] * limbs_per);
@@ -1437,7 +1442,10 @@ tn_status tn_count_batch(tn_ctx *ctx, int32_t B, const float *J, const float *h,
   for (int b = 0; sat && b < B; ++b)
     if (res[b] >= kSaturated) over.push_back(b);
   if (over.empty()) return s;
-  s = count_residues(ctx, over, J, h, on_device, rep, limbs, limbs_per, E, status);
+  raw.resize(over.size() * 4);
+  res.resize(over.size() * rep.P);
+  s = queue_residues(ctx, over, J, h, on_device, rep, raw.data(), res.data());
+  s = finish_residues(ctx, s, over, rep, raw.data(), res.data(), limbs, limbs_per, E, status);
   return s != TN_OK ? s : first_of(status, B);
 }
 
@@ -1530,6 +1538,12 @@ tn_status tn_batch_run(int32_t B, tn_ctx *const *ctxs, double *E, uint64_t *limb
     uint64_t *res = nullptr;
     bool sat = false;
     std::vector<float> J, h;   // the group's couplings
+    bool counted = false;
+    std::vector<uint64_t> limbs;   // its results
+    std::vector<double> E;
+    std::vector<int32_t> status;
+    std::vector<int> over;     // instances that run again with residues, and their status
+    tn_status over_s = TN_OK;
     tn_status s = TN_OK;
   };
   std::vector<Run> runs(groups.size());
@@ -1575,37 +1589,48 @@ tn_status tn_batch_run(int32_t B, tn_ctx *const *ctxs, double *E, uint64_t *limb
     if (r.s == TN_OK) r.s = run_program(r.owner, *r.p, 0, -1, ra);
     if (r.s == TN_OK) r.s = stage_results(r.owner, *r.p, G, r.sat ? 1 : P, r.raw, r.res);
   }
+  // the saturated instances of every group are queued again before any of them is waited for
+  for (size_t gi = 0; gi < groups.size(); ++gi) {
+    Run &r = runs[gi];
+    tn_ctx *ctx = r.owner;
+    const int G = (int)groups[gi].size();
+    if (ctx->stream != r.orig) {
+      cudaError_t e = cudaStreamSynchronize(ctx->stream);
+      if (e != cudaSuccess && r.s == TN_OK)
+        r.s = fail(ctx, TN_ECUDA, std::string("batch group: ") + cudaGetErrorString(e));
+    }
+    r.E.resize(G);
+    r.status.assign(G, TN_OK);
+    if (r.s != TN_OK || !limbs) continue;
+    r.counted = true;
+    r.limbs.resize((size_t)G * limbs_per);
+    int big = 0;
+    r.s = finish_counts(ctx, G, rep, r.raw, r.res, r.limbs.data(), limbs_per, r.E.data(),
+                        r.status.data(), &big, r.sat);
+    note_counts(ctx, big, G);
+    for (int g = 0; r.sat && g < G; ++g)
+      if (r.res[g] >= kSaturated) r.over.push_back(g);
+    if (!r.over.empty())
+      r.over_s = queue_residues(ctx, r.over, r.J.data(), r.h.empty() ? nullptr : r.h.data(), 0,
+                                rep, r.raw, r.res);
+  }
   for (size_t gi = 0; gi < groups.size(); ++gi) {
     const std::vector<int> &ids = groups[gi];
     Run &r = runs[gi];
     const int G = (int)ids.size();
-    if (r.owner->stream != r.orig) {
-      tn_ctx *ctx = r.owner;
-      cudaError_t e = cudaStreamSynchronize(ctx->stream);
-      ctx->stream = r.orig;
-      if (e != cudaSuccess && r.s == TN_OK)
-        r.s = fail(ctx, TN_ECUDA, std::string("batch group: ") + cudaGetErrorString(e));
-    }
-    std::vector<double> Eg(G);
-    std::vector<int32_t> sg(G, TN_OK);
+    std::vector<double> &Eg = r.E;
+    std::vector<int32_t> &sg = r.status;
     tn_status s = r.s;
-    if (s == TN_OK && limbs) {
-      std::vector<uint64_t> lg((size_t)G * limbs_per);
-      int big = 0;
-      s = finish_counts(r.owner, G, rep, r.raw, r.res, lg.data(), limbs_per, Eg.data(), sg.data(),
-                        &big, r.sat);
-      note_counts(r.owner, big, G);
-      std::vector<int> over;
-      for (int g = 0; r.sat && g < G; ++g)
-        if (r.res[g] >= kSaturated) over.push_back(g);
-      if (!over.empty()) {
-        count_residues(r.owner, over, r.J.data(), r.h.empty() ? nullptr : r.h.data(), 0, rep,
-                       lg.data(), limbs_per, Eg.data(), sg.data());
-        s = first_of(sg.data(), G);
-      }
+    if (!r.over.empty()) {
+      finish_residues(r.owner, r.over_s, r.over, rep, r.raw, r.res, r.limbs.data(), limbs_per,
+                      Eg.data(), sg.data());
+      s = first_of(sg.data(), G);
+    }
+    r.owner->stream = r.orig;
+    if (r.counted) {
       for (int g = 0; g < G; ++g)
-        std::copy(lg.begin() + (size_t)g * limbs_per, lg.begin() + (size_t)(g + 1) * limbs_per,
-                  limbs + (int64_t)ids[g] * limbs_per);
+        std::copy(r.limbs.begin() + (size_t)g * limbs_per,
+                  r.limbs.begin() + (size_t)(g + 1) * limbs_per, limbs + (int64_t)ids[g] * limbs_per);
     } else if (s == TN_OK) {
       for (int g = 0; g < G; ++g) Eg[g] = root_energy(r.owner, r.raw + 4 * g);
     } else {

@@ -86,3 +86,33 @@ def test_a_minority_of_large_instances_stays_with_the_saturating_run(monkeypatch
     for (Ek, ck, sk), k in out:
         assert list(ck) == list(counts) and np.array_equal(Ek, E) and np.array_equal(sk, status)
         assert k > res
+
+
+def test_saturated_instances_of_many_groups_run_together(monkeypatch):
+    """tn_batch_run: lattices of eight sizes, one of each size with 60% of its bonds cut.
+    The re-runs of all groups are in flight together, in the groups' staging; energies,
+    counts and statuses (some counts are beyond the primes' range) are those of the residue
+    planes, in the first call and in the next ones."""
+    insts = []
+    for s in range(15, 23):
+        a = [I.square_lattice(s, coupling="pm1", seed=s + k) for k in range(6)]
+        J = np.array(a[0]["J"])
+        J[: len(J) * 3 // 5] = 0
+        insts += [dict(a[0], J=J)] + a[1:]
+    sgs = [P.SpinGlass(x, order="sweep", seq=I.square_sweep_order(int(round(x["n"] ** 0.5))))
+           for x in insts]
+
+    def batch():
+        st, E, counts, status = B.tn_batch_run([g.ctx for g in sgs], limbs_per=8)
+        return st, list(E), list(counts), list(status)
+
+    got = [batch() for _ in range(3)]
+    monkeypatch.setenv("TN_COUNT_RESIDUES", "1")
+    ref = batch()
+    big = [s != B.TN_OK or c >= 1 << 59 for s, c in zip(ref[3], ref[2])]
+    assert big == [k % 6 == 0 for k in range(len(insts))]
+    assert ref[0] == B.TN_EOVERFLOW and ref[3].count(B.TN_EOVERFLOW) < 8
+    for g in got:
+        assert g == ref
+    for g in sgs:
+        g.close()

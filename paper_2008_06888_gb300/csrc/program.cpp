@@ -1361,18 +1361,24 @@ struct Builder {
 
   // ---- runs of small steps (SmallRun)
   //
-  // A step counts as small up to kSmallWork products: at that size one block takes
-  // about as long as a kernel launch (~2 us).
-  static constexpr int64_t kSmallWork = 4096;
+  // A step counts as small up to kSmallWork products and kSmallOut outputs.  Its outputs are
+  // spread over one block's 512 threads, and a thread takes them one after another: two cost
+  // less than a launch of their own (about 2 us), four and more cost up to 5 us.  With 4096
+  // outputs as the limit a greedy 16 x 16 lattice took 595 us, without runs 520, now 458;
+  // a 3 x 4 x 5 lattice 259, 194 and 177; an 11 x 11 one in rows 376, 372 and 215.  Few
+  // outputs with many products stay in: 1024 products as the limit splits the runs of a
+  // greedy 10 x 10 lattice (88 -> 100 us, its count 368 -> 442).
+  static constexpr int64_t kSmallWork = 4096, kSmallOut = 1024;
   bool small_step(const Op &op) const {
     if (op.kind == OP_GATE) {
       const GateParams &g = pr.gates[op.idx];
-      return g.outer * g.Ks * g.Ns <= kSmallWork;
+      return g.outer * g.Ns <= kSmallOut && g.outer * g.Ks * g.Ns <= kSmallWork;
     }
-    if (op.kind == OP_PERM) return pr.perms[op.idx].total <= kSmallWork && pr.perms[op.idx].r <= 14;
+    if (op.kind == OP_PERM) return pr.perms[op.idx].total <= kSmallOut && pr.perms[op.idx].r <= 14;
     if (op.kind == OP_GEMM) {
       const GemmParams &g = pr.gemms[op.idx];
-      return g.K <= 64 && g.batch * g.M * g.N * g.K <= kSmallWork;
+      const int64_t out = g.batch * g.M * g.N;
+      return g.K <= 64 && out <= kSmallOut && out * g.K <= kSmallWork;
     }
     return false;
   }

@@ -286,7 +286,9 @@ tn_status tn_profile_get(tn_ctx *ctx, int32_t kind, int64_t *launches, double *m
 tn_status tn_profile_reset(tn_ctx *ctx);
 
 /* Statistics of the current plan (any pointer may be NULL): number of
- * pairwise steps, transposes, device arena bytes for energy / config / count. */
+ * pairwise steps, transposes, device arena bytes for energy / config / count
+ * (one instance; count: with the planes of 3 primes + witness, which a count
+ * of 2^59 and more needs, or of the saturating run if that needs more). */
 tn_status tn_plan_info(const tn_ctx *ctx, int32_t *n_steps, int32_t *n_transposes,
                        int64_t *arena_energy, int64_t *arena_config, int64_t *arena_count);
 

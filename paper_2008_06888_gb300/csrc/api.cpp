@@ -1706,12 +1706,17 @@ tn_status tn_plan_info(const tn_ctx *ctx, int32_t *n_steps, int32_t *n_transpose
     *arena_config = pc.arena_bytes;
   }
   if (arena_count) {
+    // the larger of the two programs a count may run: a count of 2^59 and more needs the
+    // residue planes, whichever it starts with
     const CountRep rep = count_rep(3);
-    const bool sat = sat_first(ctx);
-    if (!build_program(ctx->net, ctx->plan, PM_COUNT, ctx->dt, sat ? 1 : rep.P, 0, &pn, &err,
-                       sat ? 8 : rep.rb, sat))
+    if (!build_program(ctx->net, ctx->plan, PM_COUNT, ctx->dt, rep.P, 0, &pn, &err, rep.rb))
       return TN_EINVAL;
     *arena_count = pn.arena_bytes;
+    if (!residues_forced()) {
+      if (!build_program(ctx->net, ctx->plan, PM_COUNT, ctx->dt, 1, 0, &pn, &err, 8, true))
+        return TN_EINVAL;
+      *arena_count = std::max(*arena_count, pn.arena_bytes);
+    }
   }
   return TN_OK;
 }

@@ -929,7 +929,7 @@ tn_status tn_order(tn_ctx *ctx, int32_t method, const int32_t *seq, int32_t seq_
     auto score = [&](const Plan &pl) -> double {
       Program pg;
       std::string e2;
-      if (!build_program(ctx->net, pl, PM_ENERGY, dt, 0, 0, &pg, &e2, 8, false, false))
+      if (!build_program(ctx->net, pl, PM_ENERGY, dt, 0, 0, &pg, &e2, 8, false, false, true))
         return INFINITY;
       double tsec = 0;
       for (const Op &op : pg.ops) {
@@ -1769,9 +1769,14 @@ tn_status tn_energy_noalloc(tn_ctx *ctx, const float *J_dev, const float *h_dev,
     std::string err;
     // (its steps travel as kernel parameters: no runs, whose descriptors would need
     // device memory)
-    if (!build_program(ctx->net, ctx->plan, PM_ENERGY, ctx->dt, 0, 0, pg.get(), &err, 8, false,
-                       false))
-      return fail(ctx, TN_EINVAL, err);
+    // (q = 3: chains of shorter tiles where those of eight legs miss the scratch; their
+    // arenas differ by some hundred bytes)
+    for (bool scoring : {false, true}) {
+      if (!build_program(ctx->net, ctx->plan, PM_ENERGY, ctx->dt, 0, 0, pg.get(), &err, 8, false,
+                         false, scoring))
+        return fail(ctx, TN_EINVAL, err);
+      if (pg->arena_bytes <= (int64_t)noalloc_scratch_bytes()) break;
+    }
     ctx->prog_noalloc = std::move(pg);
     ctx->noalloc_fp = fp;
   }

@@ -236,7 +236,7 @@ struct Builder {
   // nothing from unit inputs: outer products and Hadamard-type steps)
   std::vector<char> unit;
 
-  bool small_runs = true;
+  bool small_runs = true, scoring = false;
 
   Builder(const Net &n, const Plan &p, Program &r)
       : net(n), plan(p), pr(r), q(r.q), P(r.P), rb(r.rbytes), order(p.legset.size()),
@@ -1490,7 +1490,7 @@ struct Builder {
     // q = 3 tiles: 8 legs (26 KB, two of them staged per block, four blocks per SM) of
     // which 4 are the fastest, for runs of 81 elements; 7 with the counts' planes, and
     // where programs are only scored (the order search ranks orders as it always has)
-    if (q == 3) { tmax = P == 0 && small_runs ? 8 : 7; wlow = 4; }
+    if (q == 3) { tmax = P == 0 && !scoring ? 8 : 7; wlow = 4; }
     emit_leaves();
     if (!forward()) return false;
     pr.root = loc[plan.root];
@@ -1798,7 +1798,7 @@ static SmallBody small_body(const Program &pr, const Op &op) {
 
 bool build_program(const Net &net, const Plan &plan, ProgMode mode, Dtype dt, int P,
                    int64_t seg_bytes, Program *pr, std::string *err, int rbytes, bool sat,
-                   bool small_runs) {
+                   bool small_runs, bool scoring) {
   *pr = Program();
   pr->mode = mode;
   pr->dt = dt;
@@ -1816,6 +1816,7 @@ bool build_program(const Net &net, const Plan &plan, ProgMode mode, Dtype dt, in
   pr->sat = sat;
   Builder bd(net, plan, *pr);
   bd.small_runs = small_runs;
+  bd.scoring = scoring;
   if (!bd.build(mode, seg_bytes)) {
     *err = bd.err.empty() ? "program: lowering failed" : bd.err;
     return false;

@@ -121,10 +121,11 @@ struct Program {
 // rbytes: bytes of one residue of the counting planes (8: 61-bit primes; 4:
 // 31-bit primes, the one-prime-per-pass counts).  sat (PM_COUNT, P = 1, rbytes
 // = 8): the plane holds exact, saturating counts.  small_runs: group the small
-// steps of the forward pass into runs (value and exact-count programs).
+// steps of the forward pass into runs (value and exact-count programs).  scoring: the
+// program is not run but ranks an order in the search (no runs either).
 bool build_program(const Net &net, const Plan &plan, ProgMode mode, Dtype dt, int P,
                    int64_t seg_bytes, Program *pr, std::string *err, int rbytes = 8,
-                   bool sat = false, bool small_runs = true);
+                   bool sat = false, bool small_runs = true, bool scoring = false);
 
 int64_t abs_off(const Program &pr, const Loc &l);  // arena byte offset of values
 

@@ -133,7 +133,8 @@ cudaError_t launch_frontier_sample(const FrontierPlan &p, const FrontierStep *st
 // words): {steps, levels}, level starts [levels + 1], outputs of each level, per step its
 // first output within its level, per step the word of its body, then the bodies: 64-bit
 // offsets of the values of A, B (-1: none) and C (-1: not stored) in elements and of their
-// counts in 8-byte words, digits, K, N, unit B counts, shared-memory elements of A, B and C
+// counts in 8-byte words, digits, K, N, flags (1: B counts 1; 2, 4: the rule for NaN),
+// shared-memory elements of A, B and C
 // (-1: not there), then (size, stride in A, stride in B) of each outer digit (slowest
 // first), (offset in A, in B) of each k, the offset in B of each n (N > 1).  words is a
 // multiple of 4; scratch: shared-memory elements.  sat: one plane of saturating 64-bit

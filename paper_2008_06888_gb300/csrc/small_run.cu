@@ -23,7 +23,8 @@ namespace {
 constexpr int kSmallThreads = 512;
 // words of a body before its digit and offset tables
 enum { W_A = 0, W_B = 2, W_C = 4, W_NA = 6, W_NB = 8, W_NC = 10, W_SEG = 12, W_K = 13, W_N = 14,
-       W_UNIT = 15, W_SA = 16, W_SB = 17, W_SC = 18, W_TAB = 19 };
+       W_FLAGS = 15, W_SA = 16, W_SB = 17, W_SC = 18, W_TAB = 19 };
+enum { F_UNIT = 1, F_KEEP = 2, F_LOW = 4 };
 
 __device__ __forceinline__ int64_t word64(const int32_t *w) {
   return (int64_t)((uint64_t)(uint32_t)w[0] | ((uint64_t)(uint32_t)w[1] << 32));
@@ -36,6 +37,7 @@ struct Item {
   const uint64_t *nA, *nB;       // nB: nullptr when B's counts are all 1
   const int32_t *kt;             // (kA, kB) of each k
   int Ks;
+  int flags;
   T *C, *sC;                     // global and staged copy (either may be nullptr)
   uint64_t *nC, *snC;
 };
@@ -90,7 +92,8 @@ __global__ void __launch_bounds__(kSmallThreads) k_small(const int32_t *__restri
     }
     const int64_t offB = word64(b + W_B), offC = word64(b + W_C);
     const int sa = b[W_SA], sb = b[W_SB], sc = b[W_SC];
-    const bool mul = CNT && offB >= 0 && !b[W_UNIT];
+    const bool mul = CNT && offB >= 0 && !(b[W_FLAGS] & F_UNIT);
+    w.flags = b[W_FLAGS];
     w.A = (sa >= 0 ? sX + sa : X + word64(b + W_A)) + oa;
     w.B = offB < 0 ? nullptr : (sb >= 0 ? sX + sb : X + offB) + ob;
     w.nA = !CNT ? nullptr : (sa >= 0 ? sN + sa : N + word64(b + W_NA)) + oa;
@@ -101,6 +104,9 @@ __global__ void __launch_bounds__(kSmallThreads) k_small(const int32_t *__restri
     w.snC = !CNT || sc < 0 ? nullptr : sN + sc + out;
     return w;
   };
+  // Couplings near the type's largest value overflow to infinities, whose differences are
+  // NaN.  Steps keep the rule of their own kernels: a maximum passes NaN over, in the generic
+  // gate's steps (F_KEEP) only behind the first term, and a GEMM's (F_LOW) starts at -inf.
   auto run = [&](const Item<T> &w) {
     T best = w.A[w.kt[0]];
     if (w.B != nullptr) best = best + w.B[w.kt[1]];
@@ -109,16 +115,21 @@ __global__ void __launch_bounds__(kSmallThreads) k_small(const int32_t *__restri
       cnt = w.nA[w.kt[0]];
       if (w.nB != nullptr) cnt = mulsat64(cnt, w.nB[w.kt[1]]);
     }
+    if (best != best && (w.flags & F_LOW)) {
+      best = (T)-INFINITY;
+      cnt = 0;
+    }
 #pragma unroll 4
     for (int k = 1; k < w.Ks; ++k) {
       T v = w.A[w.kt[2 * k]];
       if (w.B != nullptr) v = v + w.B[w.kt[2 * k + 1]];
+      const bool gt = v > best || (best != best && !(w.flags & F_KEEP));
       if (CNT) {
         uint64_t c = w.nA[w.kt[2 * k]];
         if (w.nB != nullptr) c = mulsat64(c, w.nB[w.kt[2 * k + 1]]);
-        cnt = v > best ? c : (v == best ? addsat64(cnt, c) : cnt);
+        cnt = gt ? c : (v == best ? addsat64(cnt, c) : cnt);
       }
-      if (v > best) best = v;
+      if (gt) best = v;
     }
     if (w.C != nullptr) *w.C = best;
     if (w.sC != nullptr) *w.sC = best;

@@ -34,6 +34,13 @@ __device__ __forceinline__ uint32_t value_key(float x) {
 }
 __device__ __forceinline__ uint32_t value_key(int32_t x) { return (uint32_t)x ^ 0x80000000u; }
 
+// A search compares each value with the best before it, so NaN (from couplings that
+// overflow) is never taken but as the first state, which it stays.
+template <typename T>
+__device__ __forceinline__ uint32_t state_key(T v, int64_t k) {
+  return v == v ? value_key(v) : k == 0 ? 0xffffffffu : 0u;
+}
+
 // OR over the warp of a 64-bit word per lane (offsets are sums of distinct powers of two)
 __device__ __forceinline__ int64_t or64(int64_t x) {
   const uint32_t lo = __reduce_or_sync(0xffffffffu, (uint32_t)x);
@@ -91,7 +98,7 @@ __device__ __forceinline__ void walk_plain(const int32_t *r, const T *X, int8_t 
     k_offsets(kl, nk, k, &oa, &ob);
     T v = A[oa];
     if (offB >= 0) v = v + B[ob];
-    const uint32_t kv = value_key(v);
+    const uint32_t kv = state_key(v, k);
     if (kv > key || (kv == key && (uint32_t)k < bk)) {   // the first k of the largest value
       key = kv;
       bk = (uint32_t)k;
@@ -282,7 +289,7 @@ __global__ void __launch_bounds__(256) k_walk_big(const int32_t *__restrict__ re
     T v = A[oa];
     if (offB >= 0) v = v + B[ob];
     const unsigned long long key =
-        ((unsigned long long)value_key(v) << 32) | (0xffffffffu - (uint32_t)k);
+        ((unsigned long long)state_key(v, k) << 32) | (0xffffffffu - (uint32_t)k);
     top = max(top, key);
   }
 #pragma unroll

@@ -15,6 +15,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "kernels.h"
 #include "chain_dev.cuh"
@@ -94,8 +95,17 @@ __global__ void __launch_bounds__(kThreads, blocks_per_sm(NG, CNT)) k_gate_sum(c
 #pragma unroll
       for (int g = 0; g < NG; ++g) {
         const T x = a[g][0] + b[g][0][j], y = a[g][1] + b[g][1][j];
-        v[g] = max(x, y);
-        if (CNT) c[g] = x > y ? na[g][0] : (x < y ? na[g][1] : addsat64(na[g][0], na[g][1]));
+        // NaN terms (couplings that overflow) as in the separate steps: values keep a first
+        // one, counting steps take maxima and count the terms that equal them
+        if constexpr (!CNT) {
+          v[g] = y > x ? y : x;
+        } else {
+          v[g] = max(x, y);
+          if constexpr (std::is_floating_point<T>::value)
+            c[g] = addsat64(x == v[g] ? na[g][0] : 0, y == v[g] ? na[g][1] : 0);
+          else
+            c[g] = x > y ? na[g][0] : (x < y ? na[g][1] : addsat64(na[g][0], na[g][1]));
+        }
       }
       if constexpr (NG == 2) {
         out[j] = v[0] + v[1];

@@ -256,8 +256,12 @@ __global__ void __launch_bounds__(256) k_gate_t(const GateParams p, const T *__r
         const I b = ob[u] + (I)p.nB[n];
         T best = a[u][0] + (p.hasB ? B[b + kB[0]] : T(0));
 #pragma unroll
-        for (int k = 1; k < KS; ++k)
-          best = max(best, a[u][k] + (p.hasB ? B[b + kB[k]] : T(0)));
+        for (int k = 1; k < KS; ++k) {
+          const T v = a[u][k] + (p.hasB ? B[b + kB[k]] : T(0));
+          // a NaN first term (couplings that overflow) stays in wide steps, as in k_gate
+          if constexpr (NS == 16) best = v > best ? v : best;
+          else best = max(best, v);
+        }
         return best;
       };
       if constexpr (VC) {

@@ -469,7 +469,7 @@ def measure_mixed(n_inst, steps, warmup, plain=True):
     return {
         "value": len(insts) / dt, "unit": "instances/s",
         "workload": f"{len(insts)} +-J square lattices, L uniform in 8..20 (base seed 2026), "
-                    f"row-by-row order, E_min + exact count (3 primes + witness), grouped "
+                    f"row-by-row order, E_min + exact count (range of 3 primes + witness), grouped "
                     f"batches through tn_batch_run",
         "ms_per_batch": dt * 1e3, "steps": steps, "instances_ok": ok,
         "unbatched_instances_per_s": 1.0 / dt1, "unbatched_sample": len(sub),
@@ -569,8 +569,8 @@ def run_ensemble(args):
 
         desc = (f"cubic 6x6x6 open Ising glass (216 spins, 540 bonds), greedy order (seed "
                 f"{ORDER_SEED}, 4096 restarts); value: J~N(0,1) fp32, h=0, E_min + sigma* per "
-                f"instance, batch {Bsz}; other: +-J, E_min + exact count (3 primes + witness), "
-                f"batch {Bc}")
+                f"instance, batch {Bsz}; other: +-J, E_min + exact count (range of 3 primes + "
+                f"witness), batch {Bc}")
         other_key = "pm_count"
     else:
         Bsz = args.batch if args.batch != 48 else 16
@@ -680,9 +680,9 @@ def run_ensemble(args):
 
 def run_chimera(args):
     """Chimera L x L K_{4,4} cells (L = 8: 512 spins, 1472 couplers), +-J, h = 0, cell-row
-    order: E_min and the exact ground-state count with 3 primes' range (at L = 8 the 61-bit
-    planes would need ~1.1 TB, so the count runs in 31-bit passes: 6 + a witness), and the
-    residual entropy ln(count) / N.  Instances one after another (seeds 1..steps)."""
+    order: E_min and the exact ground-state count with 3 primes' range (in one plane of 64-bit
+    integers where the count stays below 2^59; at L = 8 residue planes would not fit, and
+    larger counts run in 31-bit passes: 6 + a witness), and the residual entropy ln(count) / N.  Instances one after another (seeds 1..steps)."""
     import torch
     import instances as I
     import paper_2008_06888_gb300 as P
@@ -717,14 +717,13 @@ def run_chimera(args):
         "higher_is_better": True, "dtype": "int32", "data": "synthetic",
         "config": {"workload": f"chimera {L8}x{L8} K44 cells ({8 * L8 * L8} spins), +-J, h=0, "
                                f"cell-row order; E_min + exact count (range of 3 61-bit "
-                               f"primes; in 31-bit passes when their planes do not fit) per "
-                               f"instance"},
+                               f"primes) per instance"},
         "instances": rows, "clocks": clk}), flush=True)
 
 
 def run_sample(args):
-    """Uniform ground-state samples (tn_sample) of a degenerate 16x16 +-J lattice:
-    256 steps, each one batched count of 2 x 16 pinned instances."""
+    """Uniform ground-state samples (tn_sample) of a degenerate 16x16 +-J lattice: tables of
+    exact counts along one frontier sweep, then one draw per sample and spin."""
     import torch
     import instances as I
     import paper_2008_06888_gb300 as P
@@ -732,7 +731,7 @@ def run_sample(args):
     inst = I.square_lattice(16, coupling="pm1", seed=3)
     sg = P.SpinGlass(inst, order="greedy", seed=ORDER_SEED, restarts=1024)
     count, ln, E = sg.count(3)
-    sg.sample(2, seed=0)            # builds the pinned program and its graphs
+    sg.sample(2, seed=0)            # allocates the tables
     S = 16
     torch.cuda.synchronize()
     t0 = time.perf_counter()
@@ -747,7 +746,7 @@ def run_sample(args):
         "dtype": "int32",
         "config": {"workload": "square16x16 open +-J Ising glass (seed 3), greedy order; "
                                "16 samples per call, each spin fixed by its conditional "
-                               "probability from exact counts (3 primes + witness)",
+                               "probability from exact counts",
                    "log2_peak_elements": sg.log2_peak},
         "ground_states": str(count), "E_min": E, "distinct_in_last_call": distinct,
         "ms_per_call": dt * 1e3}), flush=True)

@@ -210,10 +210,17 @@ tn_status tn_count(tn_ctx *ctx, int32_t n_primes, uint64_t *limbs, int32_t *n_li
  * tn_sample -- n_samples ground states drawn uniformly at random (Sec. III:
  *   fix the spins one at a time in `order`, each with its conditional
  *   probability of being in a ground state given the spins fixed before it).
- *   The conditional probabilities are exact ratios of degeneracy counts: a
+ *   The conditional probabilities are exact ratios of degeneracy counts.  One
+ *   sweep from the last spin of `order` to the first tabulates the value and
+ *   number of the best completions for every state of the spins that still
+ *   have neighbours to come, and a draw reads two entries per spin.  The
+ *   tables (12 bytes per state and spin; up to 64 MB stay with the context)
+ *   take at most a quarter of the free device memory.  Where they would take
+ *   more, or more work than counts, for 2^59 ground states and more, and with
+ *   TN_COUNT_RESIDUES / _61 / _PASSES, the prefixes are counted instead: a
  *   unit field on each fixed spin selects, among the ground states, those
- *   that agree with it, and tn_count_batch counts them (3 primes + witness),
- *   two candidates per sample and step, 16 samples per batch; n_spins steps.
+ *   that agree with it, and tn_count_batch counts them, two candidates per
+ *   sample and step, 16 samples per batch; n_spins steps.  Same samples.
  *   order: n_spins distinct spin ids, or NULL for 0..n_spins-1.  seed: sample
  *   s draws from a counter-based generator keyed by (seed, s, step), so the
  *   result does not depend on n_samples.  sigma: n_samples * n_spins values
@@ -297,7 +304,8 @@ tn_status tn_plan_info(const tn_ctx *ctx, int32_t *n_steps, int32_t *n_transpose
  *   (host only; Sec. III: which steps run as transposes + GEMMs and which as
  *   gate contractions or fused chains).  mode: 0 tn_energy, 1 tn_config
  *   (checkpoints kept, traceback included), 2 tn_count with 3 primes +
- *   witness.  counts: 7 int64 entries, indexed by the kinds of
+ *   witness: the program that the context's next count starts with (see
+ *   tn_count).  counts: 7 int64 entries, indexed by the kinds of
  *   tn_profile_get (a counting GEMM or transpose is two launches: values and
  *   residue planes).  Errors: TN_EINVAL (arguments), TN_ESTATE (no order).
  */

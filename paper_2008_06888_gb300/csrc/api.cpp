@@ -1731,8 +1731,8 @@ tn_status tn_plan_launches(const tn_ctx *ctx, int32_t mode, int64_t *counts) {
   if (!build_program(ctx->net, ctx->plan, pm, ctx->dt, pm == PM_COUNT ? rep.P : 0, 0, &pg, &err,
                      pm == PM_COUNT ? rep.rb : 8))
     return TN_EINVAL;
-  // counts run with one plane of exact integers first where they are likely to fit
-  // (the residue program above is then the one that saturated counts run on)
+  // the program that the next count starts with: one plane of exact integers, unless the
+  // residue program above, which saturated counts run (a program dump lists both)
   if (pm == PM_COUNT && sat_first(ctx) &&
       !build_program(ctx->net, ctx->plan, pm, ctx->dt, 1, 0, &pg, &err, 8, true))
     return TN_EINVAL;

@@ -6,7 +6,8 @@
 // 4-byte residue planes of the modular counts.  One pass then moves (4 + 8) bytes per
 // element each way for up to four replaced legs, where the residue form moves (4 + 28)
 // for three.  A replace gate costs about 10 instructions per state (two sums, a
-// maximum, two comparisons, the selection of the 64-bit count, half of its sum).
+// maximum, two comparisons, the selection of the 64-bit count, half of its sum).  Five
+// blocks of 128 threads per SM leave 96 registers a thread: every form spills 8 to 64 bytes.
 //
 // Gate counts: a leaf operand counts 1 everywhere, so a table gate made of leaves
 // only selects and adds the states' counts; otherwise its count table (the product

@@ -189,9 +189,9 @@ tn_status tn_gradient(tn_ctx *ctx, float *dJ, float *dh, int32_t on_device);
  *   n_primes in [1, 8] sets the range: the count is exact up to about
  *   2^(61*n_primes).  Counts below 2^59 need no residues: the first run keeps
  *   one 8-byte plane of exact, saturating counts, and only a count that
- *   reaches 2^59 there is run again with residue planes.  A context whose last
- *   counts did starts with the residues, until its counts are small again
- *   (before its first count the number of spins decides); TN_COUNT_RESIDUES
+ *   reaches 2^59 there is run again with residue planes.  A context most of
+ *   whose last counts did starts with the residues, until its counts are small
+ *   again (before its first count the number of spins decides); TN_COUNT_RESIDUES
  *   leaves the saturating run out.  The residues are kept modulo ceil(61*n_primes/31)
  *   31-bit primes 2^31 - c in 4-byte planes when those fit in 9 planes
  *   (n_primes <= 4; TN_COUNT_61 forces the other form), else modulo n_primes

@@ -53,7 +53,8 @@ struct tn_ctx {
   int64_t arena_cap = 0;
   std::unique_ptr<Program> prog[3];
   std::unique_ptr<Program> prog_sat;   // counts in one plane of exact 64-bit integers
-  int big_counts = -1;   // whether counts start with residues: -1 by size, else as the last did
+  int big_counts = -1;     // whether counts start with residues: -1 by size, else note_counts
+  double big_share = -1;   // share of counts of 2^59 and more, the last ones weighing most
   int prog_P = 0, prog_rb = 8;
   bool have_state = false;
   bool fwd_done = false;   // tn_forward ran last; its checkpoints are live
@@ -773,10 +774,19 @@ constexpr uint64_t kSaturated = 1ull << 59;
 // (2.5 us) is the time of 2^19 elements, so that is (3 - 1) B - 3 big elements' work below
 // 2^19.  (16 lattices of side 14, 4 or 8 of them big: 0.92 ms with residues at once, 1.27
 // with two runs; side 20, 8 big: 24.4 and 20.7; 134 lattices of side 8 to 20, 2 of them
-// big: 35.0 and 12.4.)
+// big: 35.0 and 12.4.)  A single count runs again or not, and the saturating run takes 0.2 to
+// 0.45 of the residues' time, so residues pay where about three counts in four are big.
+// The share is a running one: where couplings change between counts, the last alone is a poor
+// guess.  (16 x 16 lattices with two thirds, nine tenths and all of the counts big: 1.13, 1.31
+// and 1.44 ms with the saturating run always first, 1.16 with residues always.)
 void note_counts(tn_ctx *ctx, int big, int B) {
-  ctx->big_counts =
-      big > 0 && (2.0 * B - 3.0 * big) * std::exp2(ctx->plan.log2_peak) < (double)(1 << 19);
+  const double x = (double)big / B;
+  ctx->big_share = ctx->big_share < 0 ? x : (3 * ctx->big_share + x) / 4;
+  if (B == 1)
+    ctx->big_counts = ctx->big_share > 0.75;
+  else
+    ctx->big_counts =
+        big > 0 && (2.0 * B - 3.0 * big) * std::exp2(ctx->plan.log2_peak) < (double)(1 << 19);
 }
 bool is_big(const std::vector<uint64_t> &limbs) { return limbs.size() > 1 || limbs[0] >= kSaturated; }
 

@@ -1,6 +1,6 @@
 """Counts start the way the last ones ended: a context whose counts reach 2^59 goes to the
-residue planes at once from its second count on, and back to the saturating run when they
-are small again.  Launches tell which programs ran; counts are exact either way."""
+residue planes at once (from its second count on when the first did), and back to the
+saturating run when they are small again.  Launches tell which programs ran; counts are exact either way."""
 import numpy as np
 import pytest
 
@@ -45,13 +45,36 @@ def test_single_counts_change_their_start(monkeypatch):
     assert sat != res
     sg = _sg()
     got = []
-    for J in (BASE["J"], BASE["J"], ZERO, ZERO, ZERO, BASE["J"], BASE["J"]):
+    for J in [BASE["J"]] + [ZERO] * 7 + [BASE["J"]] * 2:
         sg.set_couplings(J)
         got.append(_launches(sg, count(sg)))
     sg.close()
-    assert [c for c, _ in got] == [want, want, 1 << 81, 1 << 81, 1 << 81, want, want]
-    # saturated: both programs; then residues; the first small count still in residues
-    assert [n for _, n in got] == [sat, sat, sat + res, res, res, res, sat]
+    assert [c for c, _ in got] == [want] + [1 << 81] * 7 + [want] * 2
+    # saturated: both programs, until the running share (1/4, 7/16, ... of the last) passes
+    # three quarters; then residues, the first small count still in them
+    assert [n for _, n in got] == [sat] + [sat + res] * 5 + [res] * 3 + [sat]
+
+
+def test_a_first_count_decides_alone(monkeypatch):
+    count = lambda sg: lambda: sg.count(3)[0]  # noqa: E731
+    sat, res = (_alone(count, r, monkeypatch) for r in (False, True))
+    sg = _sg()
+    sg.set_couplings(ZERO)
+    got = [_launches(sg, count(sg)) for _ in range(3)]
+    sg.close()
+    assert got == [(1 << 81, n) for n in (sat + res, res, res)]
+
+
+def test_one_large_count_in_three_stays_with_the_saturating_run(monkeypatch):
+    count = lambda sg: lambda: sg.count(3)[0]  # noqa: E731
+    sat, res = (_alone(count, r, monkeypatch) for r in (False, True))
+    sg = _sg()
+    got = []
+    for k in range(12):
+        sg.set_couplings(ZERO if k % 3 == 2 else BASE["J"])
+        got.append(_launches(sg, count(sg))[1])
+    sg.close()
+    assert got == [sat, sat, sat + res] * 4
 
 
 @pytest.mark.parametrize("zeros,route", [(0, "sat"), (1, "res"), (5, "res")])

@@ -1568,7 +1568,7 @@ struct SmallBody {
   int64_t offA = 0, offB = -1, offC = 0;   // element offsets of the values (B: -1 none)
   int64_t nA = 0, nB = 0, nC = 0;          // and of the counts, in 8-byte words
   int nout = 0, unitB = 1;
-  bool keep = false, low = false;          // what NaN terms do (small_run.cu)
+  bool keep = false, low = false;          // what NaN values do (small_run.cu)
   int sA = -1, sB = -1, sC = -1;           // shared-memory elements (-1: not there)
   int Ks = 1, Ns = 1;
   std::vector<int64_t> seg_size, seg_sA, seg_sB;   // outer digits, slowest first
@@ -1771,8 +1771,7 @@ static SmallBody small_body(const Program &pr, const Op &op) {
     b.Ns = g.Ns;
     b.unitB = g.unitB;
     // the forms that have kernels of their own take plain maxima
-    b.keep = !(g.Ks <= 2 && g.Ns <= 2) && !(g.Ks == 1 && g.Ns == 4) &&
-             !(pr.sat ? g.Ks == 2 && (g.Ns == 4 || g.Ns == 16) : g.Ks == 4 && g.Ns == 1);
+    b.keep = !(g.Ks <= 2 && g.Ns <= 2) && !(g.Ks == 1 && g.Ns == 4) && !(g.Ks == 4 && g.Ns == 1);
     b.nout = (int)(g.outer * g.Ns);
     b.kA.assign(g.kA, g.kA + g.Ks);
     b.kB.assign(g.kB, g.kB + g.Ks);

@@ -35,11 +35,13 @@ __device__ __forceinline__ uint32_t value_key(float x) {
 __device__ __forceinline__ uint32_t value_key(int32_t x) { return (uint32_t)x ^ 0x80000000u; }
 
 // A search compares each value with the best before it, so NaN (from couplings that
-// overflow) is never taken but as the first state, which it stays.
-template <typename T>
-__device__ __forceinline__ uint32_t state_key(T v, int64_t k) {
-  return v == v ? value_key(v) : k == 0 ? 0xffffffffu : 0u;
+// overflow) is never taken but as the first state, which it stays.  nan: the key of NaN,
+// chosen ahead of the load by the state's number.
+__device__ __forceinline__ uint32_t state_key(float x, uint32_t nan) {
+  const uint32_t key = value_key(x);
+  return x != x ? nan : key;
 }
+__device__ __forceinline__ uint32_t state_key(int32_t x, uint32_t) { return value_key(x); }
 
 // OR over the warp of a 64-bit word per lane (offsets are sums of distinct powers of two)
 __device__ __forceinline__ int64_t or64(int64_t x) {
@@ -95,10 +97,11 @@ __device__ __forceinline__ void walk_plain(const int32_t *r, const T *X, int8_t 
   uint32_t key = 0, bk = 0xffffffffu;
   for (int k = lane; k < Ks; k += 32) {
     int64_t oa, ob;
+    const uint32_t nan = k == 0 ? 0xffffffffu : 0u;
     k_offsets(kl, nk, k, &oa, &ob);
     T v = A[oa];
     if (offB >= 0) v = v + B[ob];
-    const uint32_t kv = state_key(v, k);
+    const uint32_t kv = state_key(v, nan);
     if (kv > key || (kv == key && (uint32_t)k < bk)) {   // the first k of the largest value
       key = kv;
       bk = (uint32_t)k;
@@ -289,7 +292,7 @@ __global__ void __launch_bounds__(256) k_walk_big(const int32_t *__restrict__ re
     T v = A[oa];
     if (offB >= 0) v = v + B[ob];
     const unsigned long long key =
-        ((unsigned long long)state_key(v, k) << 32) | (0xffffffffu - (uint32_t)k);
+        ((unsigned long long)state_key(v, k == 0 ? 0xffffffffu : 0u) << 32) | (0xffffffffu - (uint32_t)k);
     top = max(top, key);
   }
 #pragma unroll
